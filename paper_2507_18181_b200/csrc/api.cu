@@ -32,8 +32,7 @@ extern "C" const char* specasr_last_error(void) { return g_err; }
   } while (0)
 
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
-// Token counts are padded to 16, 32, 64, 128 or 256 so that the activation block of a projection is one TMA box
-// and one MMA (a padded count like 48 would need three narrow MMAs per k-step).
+// Workspace rows: 16, 32, 64, 128 or 256.
 static inline int pad_tokens(int n) {
   int p = 16;
   while (p < n) p <<= 1;
@@ -328,10 +327,15 @@ extern "C" specasr_status specasr_kv_create(const specasr_model* m, void* k_pool
   if (m->cfg.gemm_path == 0) {
     const specasr_model_config& c = m->cfg;
     bool ok = true;
-    for (int i = 0, b = 16; i < 5 && b <= kv->n_alloc && ok; ++i, b <<= 1) {
-      ok = make_act_map(&kv->tm_H[i], kv->ws.H, c.d_model, kv->n_alloc, b) &&
-           make_act_map(&kv->tm_AO[i], kv->ws.AO, m->q_dim, kv->n_alloc, b) &&
-           make_act_map(&kv->tm_A[i], kv->ws.A, c.ffn, kv->n_alloc, b);
+    for (int i = 0, b = 16; i < 3 && b <= kv->n_alloc && ok; ++i, b <<= 1) {
+      ok = make_act_map(&kv->tm_H[i], kv->ws.H, c.d_model, kv->n_alloc, b, 2) &&
+           make_act_map(&kv->tm_AO[i], kv->ws.AO, m->q_dim, kv->n_alloc, b, 2) &&
+           make_act_map(&kv->tm_A[i], kv->ws.A, c.ffn, kv->n_alloc, b, 2);
+    }
+    for (int i = 0; i < kActBoxes && kActBoxRows[i] <= kv->n_alloc && ok; ++i) {
+      ok = make_act_map(&kv->tm_H1[i], kv->ws.H, c.d_model, kv->n_alloc, kActBoxRows[i], 1) &&
+           make_act_map(&kv->tm_AO1[i], kv->ws.AO, m->q_dim, kv->n_alloc, kActBoxRows[i], 1) &&
+           make_act_map(&kv->tm_A1[i], kv->ws.A, c.ffn, kv->n_alloc, kActBoxRows[i], 1);
     }
     kv->attn_tc = ok && attention_tc_supported(m);
     if (kv->attn_tc) ok = attention_tc_make_maps(kv);
@@ -467,7 +471,7 @@ static void run_gemm(specasr_kv* kv, GemmArgs& a, int kind, cudaStream_t s) {
     return;
   }
 #endif
-  a.splits = gemm_tc_pick_splits(kv->m, a.M, a.K, a.n_pad);
+  a.splits = gemm_tc_pick_splits(kv->m, a.M, a.K);
   launch_gemm_tc(kv, a, kind, s);
 }
 
@@ -527,8 +531,8 @@ static void run_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int
     launch_fused_stack(m, wk, tab, n_total, n_max, ctl_shared, want_head, out_logits, want_top2, s);
     return;
   }
-  const int n_pad = pad_tokens(n);
   const bool tc = c.gemm_path == 0;
+  const int n_pad = tc ? gemm_tc_pad(n) : pad_tokens(n);
   int pending = 0;               // partial planes of the last down projection still to be added to X
   GemmArgs a;
   memset(&a, 0, sizeof(a));
@@ -539,7 +543,7 @@ static void run_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int
   a.P = wk->ws.P;
   for (int l = 0; l < c.n_layers; ++l) {
     launch_rmsnorm_split(wk, ctl_shared, m->g_attn[l], n, n_pad, pending, s);
-    a.W = m->wqkv[l]; a.tmW = tc ? &m->tm_wqkv[l] : nullptr; a.tmAct = wk->tm_H; a.act = wk->ws.H;
+    a.W = m->wqkv[l]; a.tmW = tc ? &m->tm_wqkv[l] : nullptr; a.tmAct = wk->tm_H1; a.act = wk->ws.H;
     a.M = m->qkv_dim; a.K = c.d_model; a.epilogue = EPI_PARTIAL;
     run_gemm(wk, a, SPECASR_KIND_GEMM_QKV, s);
     launch_rope_append(wk, tab, n, l, a.splits, s);
@@ -549,21 +553,21 @@ static void run_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int
 #endif
       launch_tree_attention_tc(wk, tab, n_max, l, s);
     launch_attn_merge(wk, ctl_shared, n, n_pad, tab.splits, s);
-    a.W = m->wo[l]; a.tmW = tc ? &m->tm_wo[l] : nullptr; a.tmAct = wk->tm_AO; a.act = wk->ws.AO;
+    a.W = m->wo[l]; a.tmW = tc ? &m->tm_wo[l] : nullptr; a.tmAct = wk->tm_AO1; a.act = wk->ws.AO;
     a.M = c.d_model; a.K = m->q_dim; a.epilogue = EPI_PARTIAL;
     run_gemm(wk, a, SPECASR_KIND_GEMM_O, s);
     launch_rmsnorm_split(wk, ctl_shared, m->g_ffn[l], n, n_pad, a.splits, s);
-    a.W = m->wgu[l]; a.tmW = tc ? &m->tm_wgu[l] : nullptr; a.tmAct = wk->tm_H; a.act = wk->ws.H;
+    a.W = m->wgu[l]; a.tmW = tc ? &m->tm_wgu[l] : nullptr; a.tmAct = wk->tm_H1; a.act = wk->ws.H;
     a.M = 2 * c.ffn; a.K = c.d_model; a.epilogue = EPI_SWIGLU; a.A = wk->ws.A;
     run_gemm(wk, a, SPECASR_KIND_GEMM_GU, s);
-    a.W = m->wd[l]; a.tmW = tc ? &m->tm_wd[l] : nullptr; a.tmAct = wk->tm_A; a.act = wk->ws.A;
+    a.W = m->wd[l]; a.tmW = tc ? &m->tm_wd[l] : nullptr; a.tmAct = wk->tm_A1; a.act = wk->ws.A;
     a.M = c.d_model; a.K = c.ffn; a.epilogue = EPI_PARTIAL;
     run_gemm(wk, a, SPECASR_KIND_GEMM_DOWN, s);
     pending = a.splits;
   }
   if (!want_head) return;   // context fill: K/V of every layer are written, the last FFN output is not needed
   launch_rmsnorm_split(wk, ctl_shared, m->g_final, n, n_pad, pending, s);
-  a.W = m->lm_head; a.tmW = tc ? &m->tm_lm : nullptr; a.tmAct = wk->tm_H; a.act = wk->ws.H;
+  a.W = m->lm_head; a.tmW = tc ? &m->tm_lm : nullptr; a.tmAct = wk->tm_H1; a.act = wk->ws.H;
   a.M = c.vocab; a.K = c.d_model; a.epilogue = EPI_ARGMAX; a.amax = wk->ws.amax; a.logits = out_logits;
   run_gemm(wk, a, SPECASR_KIND_GEMM_LM, s);
 }

@@ -15,6 +15,8 @@ typedef __nv_bfloat16 bf16;
 
 constexpr int kMaxSplitK = 12;     // partial planes of the linear projections
 constexpr int kMaxAttnSplits = 40; // KV splits of the attention kernels
+constexpr int kActBoxes = 7;
+constexpr int kActBoxRows[kActBoxes] = {16, 32, 64, 80, 96, 112, 128};   // token rows of a one-plane activation box
 constexpr int kCtlWords = 64;      // int32 control block at the start of the workspace
 
 // control block word indices
@@ -114,8 +116,10 @@ struct specasr_kv {
   std::vector<int> prof_kinds;
   size_t prof_used;                       // launches recorded since the last read
   TraceBuf trace;                         // device-side trace, off unless specasr_trace_set was called
-  // activation TMA descriptors (tcgen05 path), one per box height 16 << i
-  CUtensorMap tm_H[5], tm_AO[5], tm_A[5];
+  // activation TMA descriptors (tcgen05 path): boxes of both planes for the fused stack, one per height 16 << i, and
+  // boxes of one plane for the separate projections, one per height in kActBoxRows
+  CUtensorMap tm_H[3], tm_AO[3], tm_A[3];
+  CUtensorMap tm_H1[kActBoxes], tm_AO1[kActBoxes], tm_A1[kActBoxes];
   // tensor-core attention: rotated queries and the two pools
   bool attn_tc;
   CUtensorMap tm_Q, tm_K, tm_V;
@@ -167,13 +171,13 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 
 // Same, for a kernel whose CTAs form clusters of `cluster_x` along x.
 template <typename... KArgs, typename... Args>
-inline void launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster_x, cudaStream_t s,
+inline void launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster_x, size_t smem, cudaStream_t s,
                                Args&&... args) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = grid;
   cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -273,11 +277,12 @@ int gemm_fma_tiles(int M);
 void launch_gemm_fma(specasr_kv* kv, const GemmArgs& a, int kind, cudaStream_t s);
 int gemm_tc_tiles(int M);
 size_t gemm_tc_fixup_bytes(const specasr_model* m, int n_alloc);
-int gemm_tc_pick_splits(const specasr_model* m, int M, int K, int n_pad);
+int gemm_tc_pad(int n);                                       // rows a call's projections are padded to
+int gemm_tc_pick_splits(const specasr_model* m, int M, int K);
 void launch_gemm_tc(specasr_kv* kv, const GemmArgs& a, int kind, cudaStream_t s);   // a.ctl = control block to check
 bool make_tensor_map_2d(CUtensorMap* out, const void* base, uint64_t inner, uint64_t outer,
                         uint32_t box_inner, uint32_t box_outer);
-bool make_act_map(CUtensorMap* out, const void* base, uint64_t K, uint64_t n_alloc, uint32_t box_rows);
+bool make_act_map(CUtensorMap* out, const void* base, uint64_t K, uint64_t n_alloc, uint32_t box_rows, uint32_t planes);
 // bf16 tensor map of any rank with 128-byte swizzle; strides[i] is the byte stride of dimension i + 1
 bool make_tensor_map_nd(CUtensorMap* out, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
                         const uint32_t* box);

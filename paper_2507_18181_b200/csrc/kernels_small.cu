@@ -282,7 +282,7 @@ void launch_rmsnorm_split(specasr_kv* kv, const int32_t* ctl, const float* gain,
   const size_t stride = (size_t)kv->n_alloc * d;
   LaunchScope scope(kv, SPECASR_KIND_NORM, s);
 #define NORM_LAUNCH(I)                                                                                           \
-  launch_pdl_cluster(k_rmsnorm_split<I>, dim3(kNormCluster * n_pad), dim3(256), kNormCluster, s, ctl,          \
+  launch_pdl_cluster(k_rmsnorm_split<I>, dim3(kNormCluster * n_pad), dim3(256), kNormCluster, 0, s, ctl,       \
                      kv->ws.X, kv->ws.P, n_partials, stride, gain, d, d_part, m->cfg.rms_eps, n, stride, kv->ws.H \
                      SPECASR_TRACE_ARG(kv))
   if (d_part <= 1024) NORM_LAUNCH(1);

@@ -1,0 +1,30 @@
+"""Calls of more than 64 rows (separate kernels: CTA-pair projections) at the edges of their shapes: the smallest such
+call, the last split-plane one and the first folded one, row counts that are no multiple of the 32-row padding, and the
+largest.  Two shapes whose weight matrices have odd and even numbers of 128-row tiles.  Bars as in test_gpu_parity.py;
+the context fill runs through the same kernels, so its caches are compared too."""
+import numpy as np
+import pytest
+
+import gen
+from oracle import specasr_oracle as O
+from test_gpu_parity import _check_against_oracle, _fill_both, _gpu_stack, _verify_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("cfg_name,nodes", [("tiny", 65), ("tiny", 97), ("tiny", 129), ("tiny", 200), ("tiny", 256),
+                                            ("small", 96), ("small", 128), ("small", 161), ("small", 225)])
+def test_calls_of_more_than_64_rows_match_the_oracle(cfg_name, nodes):
+    cfg, store, model, kv = _gpu_stack(cfg_name, 0, 0, max_tokens=768, max_nodes=256, shuffle=3)
+    n_audio = 300 if cfg_name == "tiny" else 190           # context fill: one or two chunks, the last one ragged
+    W, cache, prompt = _fill_both(cfg, store, kv, n_audio, 4, 0)
+    for layer in (0, cfg.n_layers - 1):
+        k, v = kv.read_kv(layer, cache.length)
+        assert np.abs(k - cache.K[layer]).max() < 2e-3 and np.abs(v - cache.V[layer]).max() < 2e-3
+    parent = gen.sparse_tree(nodes, seed=nodes)
+    tokens = gen.fill_tree_tokens(parent, cfg.vocab, seed=1, root_token=int(prompt[-1]))
+    want = O.verify_tree(cfg, W, cache, tokens, parent)
+    got = _verify_gpu(cfg, kv, tokens, parent)
+    _check_against_oracle(got, want, tokens, parent)
+    again = _verify_gpu(cfg, kv, tokens, parent)
+    assert np.array_equal(again["logits"], got["logits"])
