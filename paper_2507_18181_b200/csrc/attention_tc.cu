@@ -38,6 +38,7 @@ struct AttnCtl {
   unsigned long long bar_qk, bar_v, bar_s, bar_p[2], bar_o[2];
   float red_max[2][128];      // per-row partial maxima / sums of the two warps that share a row
   float red_sum[2][128];
+  int page[KEYS_MAX / 16];    // pool page (of the layer) of every page of the key block
   uint32_t tmem_base;
   int abort;
 };
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(64 + SOFTMAX_THREADS, 1) k_tree_attention_tc(c
   extern __shared__ uint8_t smem_raw[];
   pdl_launch_dependents();
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   // grid z = utterance * (key blocks per utterance) + key block; the utterance's own values complete the parameters
   const int kvh = blockIdx.x, split = blockIdx.z % tab.splits;
   const SegDev& sg = tab.seg[blockIdx.z / tab.splits];
@@ -150,52 +151,51 @@ __global__ void __launch_bounds__(64 + SOFTMAX_THREADS, 1) k_tree_attention_tc(c
   if (!active) {
     // nothing to do for this CTA
   } else if (warp == 0) {
-    // ---------------- TMA producer: lane 0 fetches Q, lane j fetches page j of K and later of V
-    const uint32_t q_bytes = 2 * H * rows_used * 128;
-    const uint32_t kv_bytes = 2 * H * pages * p.page_size * 128;
-    if (lane == 0) {
-      mbar_expect_tx(&sc->bar_qk, q_bytes + kv_bytes);
-      mbar_expect_tx(&sc->bar_v, kv_bytes);
-    }
+    // ---------------- TMA producer: one thread issues every box
+    if (lane < pages) sc->page[lane] = p.layer * p.n_pages + my_page;
     __syncwarp();
-    if (lane == 0) {
+    if (elect_one()) {
+      const uint32_t kv_bytes = 2 * H * pages * p.page_size * 128;
+      mbar_expect_tx(&sc->bar_qk, 2 * H * rows_used * 128 + kv_bytes);
+      mbar_expect_tx(&sc->bar_v, kv_bytes);
       for (int plane = 0; plane < 2; ++plane)
         for (int h = 0; h < H; ++h)
           tma_load_4d(As + (plane * H + h) * SUB, &tmQ, h * 64, kvh * p.group, p.row0 + node0, plane, &sc->bar_qk);
+      const CUtensorMap* map = tmK;
+      void* bar = &sc->bar_qk;
+      bool ok = true;
+#pragma unroll 1
+      for (int kv = 0; kv < 2 && ok; ++kv) {
+#pragma unroll 1
+        for (int j = 0; j < pages; ++j) {
+          const int c4 = sc->page[j];
+          uint8_t* dst = KVs + j * p.page_size * 128;
+#pragma unroll
+          for (int sub = 0; sub < 2 * H; ++sub)
+            tma_load_5d(dst + sub * KVSUB, map, (sub % H) * 64, 0, sub / H, kvh, c4, bar);
+        }
+        // V takes K's place once the S MMAs have read K
+        if (kv == 0) ok = mbar_wait(&sc->bar_s, 0u, abort, status);
+        map = tmV;
+        bar = &sc->bar_v;
+      }
     }
-    int c4 = 0;
-    const int off = lane * p.page_size * 128;
-    if (lane < pages) {
-      c4 = p.layer * p.n_pages + my_page;
-      for (int plane = 0; plane < 2; ++plane)
-        for (int h = 0; h < H; ++h)
-          tma_load_5d(KVs + (plane * H + h) * KVSUB + off, tmK, h * 64, 0, plane, kvh, c4, &sc->bar_qk);
-    }
-    // V takes K's place once the S MMAs have read K
-    const bool ok = mbar_wait(&sc->bar_s, 0u, abort, status);
-    if (ok && lane < pages) {
-      for (int plane = 0; plane < 2; ++plane)
-        for (int h = 0; h < H; ++h)
-          tma_load_5d(KVs + (plane * H + h) * KVSUB + off, tmV, h * 64, 0, plane, kvh, c4, &sc->bar_v);
-    }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     // ---------------- MMA issuer
     bool ok = mbar_wait(&sc->bar_qk, 0u, abort, status);
     if (ok) {
       tc_fence_after();
       const uint32_t idesc = make_idesc_bf16(kc_pad);
-      const uint32_t a0 = smem_u32(As), b0 = smem_u32(KVs);
-      uint32_t acc = 0u;
+      const uint32_t a_lo = smem_desc_lo(smem_u32(As)), b_lo = smem_desc_lo(smem_u32(KVs));
 #pragma unroll
       for (int term = 0; term < 3; ++term) {
         const int qp = term == 2 ? 1 : 0, kp = term == 1 ? 1 : 0;     // hi*hi, hi*lo, lo*hi
+#pragma unroll
         for (int h = 0; h < H; ++h) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            umma_bf16(tmem_s, make_smem_desc(a0 + (qp * H + h) * SUB + k * 32),
-                      make_smem_desc(b0 + (kp * H + h) * KVSUB + k * 32), idesc, acc);
-            acc = 1u;
-          }
+          for (int k = 0; k < 4; ++k)
+            umma_bf16_lo(tmem_s, a_lo + (((qp * H + h) * SUB + k * 32) >> 4), b_lo + (((kp * H + h) * KVSUB + k * 32) >> 4),
+                         idesc, (term | h | k) ? 1u : 0u);
         }
       }
       umma_commit(&sc->bar_s);
@@ -207,7 +207,8 @@ __global__ void __launch_bounds__(64 + SOFTMAX_THREADS, 1) k_tree_attention_tc(c
       ok = mbar_wait(&sc->bar_p[rd], 0u, abort, status);
       if (!ok) break;
       tc_fence_after();
-      const uint32_t a0 = smem_u32(As), b0 = smem_u32(KVs);
+      const uint32_t a_lo = smem_desc_lo(smem_u32(As));
+      const uint32_t b_lo = smem_desc_lo(smem_u32(KVs), KVSUB) + (uint32_t)((rd * (ROUND / 16) * 2048) >> 4);
       const int j_end = min(kc_pad - rd * ROUND, ROUND) / 16;
 #pragma unroll
       for (int term = 0; term < 3; ++term) {
@@ -215,8 +216,8 @@ __global__ void __launch_bounds__(64 + SOFTMAX_THREADS, 1) k_tree_attention_tc(c
         for (int j = 0; j < j_end; ++j) {
           // A: P plane pp, 64-key block j / 4 of this round, 16 keys = 32 bytes along the row
           // B: V plane vp, keys of this step are rows of 128 bytes; the second half of the head is KVSUB further on
-          umma_bf16(tmem_o, make_smem_desc(a0 + (pp * 2 + (j >> 2)) * SUB + (j & 3) * 32),
-                    make_smem_desc(b0 + vp * H * KVSUB + (rd * (ROUND / 16) + j) * 2048, KVSUB), idesc2, acc);
+          umma_bf16_lo(tmem_o, a_lo + (((pp * 2 + (j >> 2)) * SUB + (j & 3) * 32) >> 4),
+                       b_lo + ((vp * H * KVSUB + j * 2048) >> 4), idesc2, acc);
           acc = 1u;
         }
       }

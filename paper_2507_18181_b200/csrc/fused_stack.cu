@@ -85,6 +85,7 @@ struct alignas(16) StackCtl {
   float red_sum[2][128];
   float inv[64];                        // 1 / rms of every token row, for the epilogue in progress
   float red[8];
+  int page[KEYS_MAX / 16];               // pool page (of the layer) of every page of the attention unit
   uint32_t tmem_base;
   int abort;
   int attn_done;                        // attention steps this CTA has finished (its ring memory is free again)
@@ -293,7 +294,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
   uint8_t* As = ring;                                   // attention: overlays the ring
   uint8_t* KVs = ring + A_BYTES;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int G = gridDim.x, cta = blockIdx.x;
   const int n_pad = p.n_pad;
   const int act_sub = n_pad * 2 * SUB_K * 2;            // both planes of one 64-wide k sub-block
@@ -338,7 +339,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
 
   if (!live) {
     // the call was refused before it started (shared status): nothing to do
-  } else if (warp == 0 && lane == 0) {
+  } else if (warp == 0 && elect_one()) {
     // =========================================================== weight producer
     // A cursor walks this CTA's (layer, projection, unit) list, which is fixed for the call, and issues the TMA loads
     // into the ring as slots come free: weights never wait for a step, so the first tiles of the next projection
@@ -418,30 +419,38 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
     }
   } else if (warp == 10) {
     // =========================================================== activation producer / attention producer
-    int it = 0;
+    int slot = 0;                                        // next ring slot
+    uint32_t ring_par = 0u;                              // parity of the ring round in progress
     bool ok = true;
     int au = 0;                                          // attention units this CTA has run
     auto stream_acts = [&](const Gemm& g, const CUtensorMap* tmAct, int ready_step) {
       if (g.u1 <= g.u0) return;
-      if (lane == 0) {
+      if (elect_one()) {
         ok = wait_word_ge(p.sync + ready_step, G, abort, status);
         fence_proxy_async_all();
         int kb = g.u0 % g.KB;
-        for (int u = g.u0; u < g.u1 && ok; ++u, ++it) {
-          const int s = it % p.stages;
-          if (!bar_wait(&sc->empty[s], (uint32_t)((it / p.stages) & 1) ^ 1u, abort, status)) {
+        int sl = slot;
+        uint32_t par = ring_par;
+        for (int u = g.u0; u < g.u1 && ok; ++u) {
+          if (!bar_wait(&sc->empty[sl], par ^ 1u, abort, status)) {
             ok = false;
             break;
           }
-          uint8_t* st = ring + (size_t)s * p.stage_bytes + W_STAGE_BYTES;
-          mbar_expect_tx(&sc->full[s], (uint32_t)act_stage);
+          uint8_t* st = ring + (size_t)sl * p.stage_bytes + W_STAGE_BYTES;
+          mbar_expect_tx(&sc->full[sl], (uint32_t)act_stage);
           for (int q = 0; q < KSUB; ++q)
-            tma_load_3d(st + q * act_sub, tmAct, (kb * KSUB + q) * SUB_K, 0, 0, &sc->full[s]);
+            tma_load_3d(st + q * act_sub, tmAct, (kb * KSUB + q) * SUB_K, 0, 0, &sc->full[sl]);
           if (++kb == g.KB) kb = 0;
+          if (++sl == p.stages) {
+            sl = 0;
+            par ^= 1u;
+          }
         }
       }
-      ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
-      it = __shfl_sync(0xFFFFFFFFu, it, 0);
+      ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
+      const int end = slot + (g.u1 - g.u0);              // the same for every lane
+      ring_par ^= (uint32_t)(end / p.stages) & 1u;
+      slot = end % p.stages;
     };
     for (int sidx = 0; sidx < n_steps && ok; ++sidx) {
       const int l = sidx / ST_PER_LAYER, st = sidx - l * ST_PER_LAYER;
@@ -451,7 +460,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
         const CUtensorMap* tmAct = gk == ST_O ? &tmAO : gk == ST_DOWN ? &tmA : &tmH;
         stream_acts(gemm_of(p, l, gk, cta, G), tmAct, sidx - 1);
       } else if (l < p.n_layers && st == ST_ATTN) {
-        // ---- attention units of this CTA: lane 0 fetches Q, lane j page j of K and later of V.
+        // ---- attention units of this CTA: one thread issues every box.
         // (Asking for the K pages of a key block inside the committed prefix before the rotary step has finished
         // made S ready 1.6 us earlier and the step no shorter; it was taken out again.)
         bool rope_seen = false;
@@ -469,56 +478,56 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
           const int pages = (kc + p.page_size - 1) / p.page_size;
           const uint32_t par = (uint32_t)(au & 1);
           ++au;
-          auto wait_rope = [&]() {
-            if (lane == 0) {
+          // A CTA that runs several units reuses the Q / P and K / V tiles and the barriers: the next unit's loads
+          // (and the arming of its barriers) wait until the workers have stored the previous unit's output.
+          if (elect_one()) {
+            if (!rope_seen) {
               ok = wait_word_ge(p.sync + sidx - 1, G, abort, status);
               fence_proxy_async_all();
             }
-            ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
-            rope_seen = true;
-          };
-          if (!rope_seen) wait_rope();
-          // A CTA that runs several units reuses the Q / P and K / V tiles and the barriers: the next unit's loads
-          // (and the arming of its barriers) wait until the workers have stored the previous unit's output.
-          if (ok && lane == 0) ok = wait_smem_ge(&sc->units_done, au - 1, abort, status);
-          ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
+            if (ok) ok = wait_smem_ge(&sc->units_done, au - 1, abort, status);
+          }
+          rope_seen = true;
+          ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
           if (!ok) break;
-          int my_page = 0;
-          if (lane < pages) my_page = sg.page_table[split * (sg.chunk / p.page_size) + lane];
-          const uint32_t q_bytes = 2 * H2 * rows_used * 128;
-          const uint32_t kv_bytes = 2 * H2 * pages * p.page_size * 128;
-          if (lane == 0) {
+          if (lane < pages) sc->page[lane] = l * sg.n_pages + sg.page_table[split * (sg.chunk / p.page_size) + lane];
+          __syncwarp();
+          if (elect_one()) {
+            const uint32_t q_bytes = 2 * H2 * rows_used * 128;
+            const uint32_t kv_bytes = 2 * H2 * pages * p.page_size * 128;
             mbar_expect_tx(&sc->bar_qk, q_bytes + kv_bytes);
             mbar_expect_tx(&sc->bar_v, kv_bytes);
-          }
-          __syncwarp();
-          const int c4 = l * sg.n_pages + my_page;
-          const int off = lane * p.page_size * 128;
-          if (lane < pages) {
-            for (int plane = 0; plane < 2; ++plane)
-              for (int h = 0; h < H2; ++h)
-                tma_load_5d(KVs + (plane * H2 + h) * KVSUB + off, sg.tmK, h * 64, 0, plane, kvh, c4, &sc->bar_qk);
-          }
-          if (lane == 0) {
             for (int plane = 0; plane < 2; ++plane)
               for (int h = 0; h < H2; ++h)
                 tma_load_4d(As + (plane * H2 + h) * SUB, &tmQ, h * 64, kvh * p.group, sg.row0 + node0, plane, &sc->bar_qk);
+            const CUtensorMap* map = sg.tmK;
+            void* bar = &sc->bar_qk;
+#pragma unroll 1
+            for (int kv = 0; kv < 2 && ok; ++kv) {
+#pragma unroll 1
+              for (int j = 0; j < pages; ++j) {
+                const int c4 = sc->page[j];
+                uint8_t* dst = KVs + j * p.page_size * 128;
+#pragma unroll
+                for (int sub = 0; sub < 2 * H2; ++sub)
+                  tma_load_5d(dst + sub * KVSUB, map, (sub % H2) * 64, 0, sub / H2, kvh, c4, bar);
+              }
+              // V takes K's place once the S MMAs have read K
+              if (kv == 0) ok = bar_wait(&sc->bar_s, par, abort, status);
+              map = sg.tmV;
+              bar = &sc->bar_v;
+            }
           }
-          // V takes K's place once the S MMAs have read K
-          ok = bar_wait(&sc->bar_s, par, abort, status);
-          if (ok && lane < pages) {
-            for (int plane = 0; plane < 2; ++plane)
-              for (int h = 0; h < H2; ++h)
-                tma_load_5d(KVs + (plane * H2 + h) * KVSUB + off, sg.tmV, h * 64, 0, plane, kvh, c4, &sc->bar_v);
-          }
-          ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
+          ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     // =========================================================== MMA issuer
-    int it = 0, seg = 0, au = 0, au2 = 0;
+    int slot = 0, seg = 0, au = 0, au2 = 0;
+    uint32_t ring_par = 0u;
     bool ok = true;
+    const uint32_t ring_lo = smem_desc_lo(smem_u32(ring)), stage_lo = (uint32_t)(p.stage_bytes >> 4);
     const uint32_t idesc = make_idesc_bf16(2 * n_pad);
     auto run_gemm = [&](const Gemm& g) {
       for (int u = g.u0; u < g.u1 && ok; ++seg) {
@@ -531,14 +540,13 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
         }
         tc_fence_after();
         const uint32_t d_addr = tmem_base + (uint32_t)(b * TM * acc_cols);
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = it % p.stages;
-          if (!bar_wait(&sc->full[s], (uint32_t)((it / p.stages) & 1), abort, status)) {
+        for (int kb = kb0; kb < kb1; ++kb) {
+          if (!bar_wait(&sc->full[slot], ring_par, abort, status)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t w_lo = smem_desc_lo(smem_u32(ring + (size_t)s * p.stage_bytes));
+          const uint32_t w_lo = ring_lo + (uint32_t)slot * stage_lo;
           const uint32_t act_lo = w_lo + (W_STAGE_BYTES >> 4);
 #pragma unroll
           for (int t = 0; t < TM; ++t) {
@@ -552,7 +560,11 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
               }
             }
           }
-          umma_commit(&sc->empty[s]);                    // arrives once these MMAs have read the stage
+          umma_commit(&sc->empty[slot]);                 // arrives once these MMAs have read the stage
+          if (++slot == p.stages) {
+            slot = 0;
+            ring_par ^= 1u;
+          }
         }
         if (ok) umma_commit(&sc->acc_full[b]);
         u += kb1 - kb0;

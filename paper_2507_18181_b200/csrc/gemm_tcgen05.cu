@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(64 + EPI_THREADS, 1) k_proj(const __grid_const
   SharedCtl* sc = (SharedCtl*)(ring + (size_t)p.stages * stage_bytes);
   bf16* epi_stage = (bf16*)(sc + 1);                      // EPI_SWIGLU: [2 planes][64 tokens][64] output tile
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int rank = (int)cluster_rank();                   // 0 = leader
   const int cta = blockIdx.x, pair = cta >> 1, G = gridDim.x >> 1;
   const int KB = p.KB;
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(64 + EPI_THREADS, 1) k_proj(const __grid_const
   volatile int* abort = &sc->abort;
   int32_t* status = p.ctl + CTL_STATUS;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0 && elect_one()) {
     // ---------------- TMA producer: this CTA's weight tile and its half of the token operand
     const int total = u1 - u0;
     const uint32_t full0 = map_to_cta(smem_u32(&sc->full[0]), 0);      // the leader's barriers
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(64 + EPI_THREADS, 1) k_proj(const __grid_const
         }
       }
     }
-  } else if (warp == 1 && lane == 0 && rank == 0) {
+  } else if (warp == 1 && rank == 0 && elect_one()) {
     // ---------------- MMA issuer of the pair
     pdl_wait();
     if (*(volatile int32_t*)status == 0) {

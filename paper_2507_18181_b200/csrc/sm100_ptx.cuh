@@ -13,6 +13,21 @@ constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;   // every wait give
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// True in one lane of the (converged) warp.  TMA loads, MMAs and commits take their operands from uniform registers;
+// under a plain `lane == 0` the compiler cannot know that a single thread is active and wraps each of them in a loop
+// over the lanes: 58 clocks per 2 KB TMA box against 21 behind elect.sync.  The warp index that selects a role has to
+// be uniform as well (warp_index).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "elect.sync _|P, 0xFFFFFFFF;\n\t"
+      "selp.u32 %0, 1, 0, P;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0); }
+
 __device__ __forceinline__ void mbar_init(void* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
 }
@@ -118,15 +133,13 @@ __device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, i
 //  - K-major operand: a row is one M/N index, 64 bf16 of K.  `lbo` is unused (1).
 //  - MN-major operand: a row is one K index, 64 bf16 of M/N; the next 64 M/N indices start `lbo`
 //    bytes further on.
-__device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr, uint32_t lbo_bytes = 16) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;       // stride byte offset between 8-row groups
-  d |= (uint64_t)1 << 46;                 // descriptor version
-  d |= (uint64_t)2 << 61;                 // SWIZZLE_128B
-  return d;
+// Descriptors are built from their low words (start address in 16-byte units | leading byte offset << 16): the high word
+// is the same for every tile here, and an operand `off` bytes further on is `lo + (off >> 4)` (shared memory ends below
+// 256 KB, so the 14-bit address field never carries).  The issuing thread spends a few instructions per MMA this way.
+__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t saddr, uint32_t lbo_bytes = 16) {
+  return ((saddr >> 4) & 0x3FFFu) | (((lbo_bytes >> 4) & 0x3FFFu) << 16);
 }
+constexpr uint32_t SMEM_DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);   // stride 1024 B, version 1, SWIZZLE_128B
 
 // Instruction descriptor of kind::f16: D fp32, A and B bf16, M = 128, N = n; b_mn_major selects an
 // MN-major B operand (A is always K-major here).
@@ -135,24 +148,6 @@ __device__ __forceinline__ uint32_t make_idesc_bf16(int n, bool b_mn_major = fal
          ((uint32_t)(128 >> 4) << 24);
 }
 
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// The same with the descriptors given by their low words (start address in 16-byte units | leading byte offset << 16):
-// the high word is the same for every tile here, and an operand `off` bytes further on is `lo + (off >> 4)` (shared
-// memory ends below 256 KB, so the 14-bit address field never carries).  The thread that issues the MMAs spends a few
-// instructions per MMA this way instead of rebuilding two 64-bit descriptors; with short MMAs (few tokens or keys)
-// that thread, not the tensor pipe, sets the pace.
-__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t saddr, uint32_t lbo_bytes = 16) {
-  return ((saddr >> 4) & 0x3FFFu) | (((lbo_bytes >> 4) & 0x3FFFu) << 16);
-}
-constexpr uint32_t SMEM_DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);   // stride 1024 B, version 1, SWIZZLE_128B
 __device__ __forceinline__ void umma_bf16_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
                                              uint32_t accumulate) {
   asm volatile(
