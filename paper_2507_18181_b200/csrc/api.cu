@@ -475,29 +475,20 @@ static void run_gemm(specasr_kv* kv, GemmArgs& a, int kind, cudaStream_t s) {
   launch_gemm_tc(kv, a, kind, s);
 }
 
-// Key blocks of the attention over `n` nodes of one utterance; `sm_budget` is the number of SMs the launch
-// should fill (all of them for a plain call, a share of them when several utterances launch back to back).
-static int attention_splits(const specasr_kv* kv, int n, int len_upper, int sm_budget, bool* use_tc, int* chunk) {
+#ifdef SPECASR_CROSSCHECK
+// Key blocks of the plain attention kernel over `n` nodes of one utterance.
+static int plain_attention_splits(const specasr_kv* kv, int n) {
   const specasr_model_config& c = kv->m->cfg;
-  *use_tc = false;
-  *chunk = 0;
-  if (kv->attn_tc) {
-    int s = 0;
-    if (attention_tc_plan(kv->m, n, len_upper + n, sm_budget, kMaxAttnSplits, &s, chunk)) {
-      *use_tc = true;
-      return s;
-    }
-  }
   const int group = c.n_heads / c.n_kv_heads;
-  const int row_tiles = (n * group + 63) / 64;
-  const int ctas = c.n_kv_heads * row_tiles;
-  int splits = (sm_budget + ctas - 1) / ctas;
-  const int by_len = (len_upper + n + 63) / 64;
+  const int ctas = c.n_kv_heads * ((n * group + 63) / 64);
+  int splits = (kv->m->n_sm + ctas - 1) / ctas;
+  const int by_len = (kv->len_upper + n + 63) / 64;
   if (splits > by_len) splits = by_len;
   if (splits > kMaxAttnSplits) splits = kMaxAttnSplits;
   if (splits < 1) splits = 1;
   return splits;
 }
+#endif
 
 // Table entry of one utterance (everything but the attention plan).
 static SegDev seg_entry(const specasr_kv* u, int row0, int n) {
@@ -523,12 +514,12 @@ static SegDev seg_entry(const specasr_kv* u, int row0, int n) {
 // control block `ctl_shared`; the rotary/append and attention kernels look up each row's utterance in the table
 // and work against its cache and control block.  With want_head the final norm, the vocabulary projection
 // and its fused per-tile argmax run as well.
-static void run_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int n_total, int n_max, bool att_tc,
+static void run_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int n_total, bool att_tc,
                       const int32_t* ctl_shared, bool want_head, float* out_logits, bool want_top2, cudaStream_t s) {
   const specasr_model_config& c = m->cfg;
   const int n = n_total;
-  if (fused_stack_supported(wk, n_total, att_tc, tab.splits)) {
-    launch_fused_stack(m, wk, tab, n_total, n_max, ctl_shared, want_head, out_logits, want_top2, s);
+  if (fused_stack_supported(wk, n_total, att_tc)) {
+    launch_fused_stack(m, wk, tab, n_total, ctl_shared, want_head, out_logits, want_top2, s);
     return;
   }
   const bool tc = c.gemm_path == 0;
@@ -551,8 +542,8 @@ static void run_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int
     if (!att_tc) launch_tree_attention(wk, l, n, tab.splits, s);      // plain kernel, single utterance only
     else
 #endif
-      launch_tree_attention_tc(wk, tab, n_max, l, s);
-    launch_attn_merge(wk, ctl_shared, n, n_pad, tab.splits, s);
+      launch_tree_attention_tc(wk, tab, l, s);
+    launch_attn_merge(wk, tab, ctl_shared, n, n_pad, s);
     a.W = m->wo[l]; a.tmW = tc ? &m->tm_wo[l] : nullptr; a.tmAct = wk->tm_AO1; a.act = wk->ws.AO;
     a.M = c.d_model; a.K = m->q_dim; a.epilogue = EPI_PARTIAL;
     run_gemm(wk, a, SPECASR_KIND_GEMM_O, s);
@@ -578,7 +569,11 @@ static SegTable single_table(specasr_kv* kv, int n, bool* att_tc) {
   memset(&t, 0, sizeof(t));
   t.count = 1;
   t.seg[0] = seg_entry(kv, 0, n);
-  t.splits = attention_splits(kv, n, kv->len_upper, kv->m->n_sm, att_tc, &t.seg[0].chunk);
+  *att_tc = kv->attn_tc;
+  if (kv->attn_tc) attention_tc_plan(kv->m, &t, &kv->len_upper);
+#ifdef SPECASR_CROSSCHECK
+  else t.splits = t.seg[0].splits = plain_attention_splits(kv, n);
+#endif
   return t;
 }
 
@@ -608,16 +603,10 @@ static specasr_status prefill_common(specasr_model* m, specasr_kv* kv, const flo
     const int chunk = n - done < kv->max_nodes ? n - done : kv->max_nodes;
     bool att_tc = false;
     const SegTable tab = single_table(kv, chunk, &att_tc);
-#ifndef SPECASR_CROSSCHECK
-    if (!att_tc) {
-      set_error("%s: a cache of %d positions needs more key blocks than the workspace holds", who, kv->len_upper + chunk);
-      return SPECASR_ERR_UNSUPPORTED;
-    }
-#endif
     launch_chain_prep(kv, chunk, done == 0, s);
     if (embeds) launch_copy_embeds(kv, embeds + (size_t)done * m->cfg.d_model, chunk, s);
     else launch_embed_tokens(kv, tab, chunk, tokens + done, s);
-    run_stack(m, kv, tab, chunk, chunk, att_tc, kv->ws.ctl, false, nullptr, false, s);
+    run_stack(m, kv, tab, chunk, att_tc, kv->ws.ctl, false, nullptr, false, s);
     launch_advance_len(kv, chunk, s);
     kv->len_host += chunk;
     kv->len_upper = kv->len_host;
@@ -668,22 +657,15 @@ static specasr_status verify_tree_impl(specasr_model* m, specasr_kv* kv, const i
   cudaStream_t s = (cudaStream_t)stream;
   bool att_tc = false;
   const SegTable tab = single_table(kv, n_nodes, &att_tc);
-#ifndef SPECASR_CROSSCHECK
-  if (!att_tc) {
-    set_error("specasr_verify_tree: a cache of %d positions needs more key blocks than the workspace holds",
-              kv->len_upper + n_nodes);
-    return SPECASR_ERR_UNSUPPORTED;
-  }
-#endif
   const bool want_top2 = out_top2_ids != nullptr;
-  if (want_top2 && !fused_stack_supported(kv, n_nodes, att_tc, tab.splits)) {
+  if (want_top2 && !fused_stack_supported(kv, n_nodes, att_tc)) {
     set_error("specasr_verify_tree_top2: the top-2 epilogue needs the fused layer stack (tensor-core attention, at most "
               "64 nodes)");
     return SPECASR_ERR_UNSUPPORTED;
   }
   launch_tree_prep(kv, tab, tokens, parent_idx, s);
   launch_embed_tokens(kv, tab, n_nodes, tokens, s);
-  run_stack(m, kv, tab, n_nodes, n_nodes, att_tc, kv->ws.ctl, true, out_logits, want_top2, s);
+  run_stack(m, kv, tab, n_nodes, att_tc, kv->ws.ctl, true, out_logits, want_top2, s);
   launch_accept(kv, tab, nullptr, tokens, parent_idx, lm_tiles_of(m), out_argmax, out_accept_len, out_path, out_bonus, s);
   if (want_top2) launch_top2_from_tiles(kv, tab, nullptr, n_nodes, lm_tiles_of(m), out_top2_ids, out_top2_probs, s);
   kv->pending_n = n_nodes;
@@ -762,10 +744,7 @@ static specasr_status verify_batch_impl(specasr_model* m, int32_t batch, specasr
   SegTable tab;
   memset(&tab, 0, sizeof(tab));
   tab.count = batch;
-  tab.splits = 1;
-  int budget = m->n_sm / batch;
-  if (budget < 1) budget = 1;
-  int n_max = 1;
+  int len_upper[SPECASR_MAX_BATCH];
   for (int b = 0; b < batch; ++b) {
     specasr_kv* u = kv[b];
     const int n_b = node_offsets[b + 1] - node_offsets[b];
@@ -780,27 +759,20 @@ static specasr_status verify_batch_impl(specasr_model* m, int32_t batch, specasr
                 tab.seg[b].capacity);
       return SPECASR_ERR_KV_CAPACITY;
     }
-    bool use_tc = false;
-    const int sp = attention_splits(u, n_b, u->len_upper, budget, &use_tc, &tab.seg[b].chunk);
-    if (!use_tc) {
-      set_error("%s: utterance %d: cache of up to %d positions needs more key blocks than the workspace holds", who, b,
-                u->len_upper + n_b);
-      return SPECASR_ERR_UNSUPPORTED;
-    }
-    if (sp > tab.splits) tab.splits = sp;
-    if (n_b > n_max) n_max = n_b;
+    len_upper[b] = u->len_upper;
   }
+  attention_tc_plan(m, &tab, len_upper);
   cudaStream_t s = (cudaStream_t)stream;
   int32_t* ctl_shared = wk->ws.ctl + kCtlBatch;
   CUDA_TRY(cudaMemsetAsync(ctl_shared, 0, sizeof(int32_t) * 4, s));
   const bool want_top2 = out_top2_ids != nullptr;
-  if (want_top2 && !fused_stack_supported(wk, total, true, tab.splits)) {
+  if (want_top2 && !fused_stack_supported(wk, total, true)) {
     set_error("%s: the top-2 epilogue needs the fused layer stack (at most 64 nodes in all)", who);
     return SPECASR_ERR_UNSUPPORTED;
   }
   launch_tree_prep(wk, tab, tokens, parent_idx, s);
   launch_embed_tokens(wk, tab, total, tokens, s);
-  run_stack(m, wk, tab, total, n_max, true, ctl_shared, true, out_logits, want_top2, s);
+  run_stack(m, wk, tab, total, true, ctl_shared, true, out_logits, want_top2, s);
   launch_accept(wk, tab, ctl_shared, tokens, parent_idx, lm_tiles_of(m), out_argmax, out_accept_len, out_path, out_bonus,
                 s);
   if (want_top2) launch_top2_from_tiles(wk, tab, ctl_shared, total, lm_tiles_of(m), out_top2_ids, out_top2_probs, s);

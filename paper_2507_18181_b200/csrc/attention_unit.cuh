@@ -1,0 +1,357 @@
+// One unit of tree-masked grouped-query attention on the 5th-generation tensor cores (sm_100a): the code of its roles,
+// shared by the fused layer stack (fused_stack.cu) and the separate attention kernel (attention_tc.cu).
+//
+// Node i sees every committed cache position [0, L) and the tree slots L + j for which j is i or an
+// ancestor of i (bit j of the node's ancestor mask): the 2-D mask of a draft token tree.
+//
+// A unit is one KV head, a tile of up to 128 query rows (row = node * group + head-in-group, so a whole query group
+// shares every K/V element that is staged) and a range of cache positions, walked in chunks of 64 keys:
+//   S = Q K^T      M = 128 rows, N = 64 keys, K = head_dim        (Q and K in shared memory, both K-major)
+//   P = exp2(S * scale - m), masked                                 (two threads per row, fp32, from TMEM)
+//   O += P V       M = 128 rows, N = head_dim, K = 64 keys         (P in TMEM, V the MN-major B operand)
+// Q, P, K and V are all carried as two bf16 planes (value ~ hi + lo); each product is three MMAs
+// (hi*hi + hi*lo + lo*hi) into the same fp32 accumulator, which keeps ~16 significant bits.
+//
+// What bounds it: the tensor pipe, 24 score MMAs of 48 clocks (N = 64 is bound by the fetch of Q from shared memory) and
+// 12 value MMAs of 64 per chunk of head_dim 128, about 1 us per 128 x 64 block, as long as the soft-max keeps under it.
+// Hence the pipeline: chunks of K and V come through one ring in the order the MMAs want them (K0, K1, V0, K2, V1,
+// ...), the scores of chunk i + 1 are issued before the values of chunk i, and P takes the place of its own S in
+// TMEM -- each thread overwrites exactly the columns it has read -- so that no probability passes through shared memory.
+// The running maximum is only a reference: it is raised, and O rescaled, when a chunk exceeds it by more than 2^8.
+// (Before, a unit was a single shot of at most 208 keys whose loads, scores, soft-max and values followed one another:
+// 82 us per layer at 256 rows on 2048 positions of the 7B shape, 44 here; 44 against 24 at 33 rows on 4096 positions, and
+// 20 against 17 at 64 rows on 1764.)
+//
+// A unit leaves an unnormalised partial (reference in log2 units, row sum, output) that the merge step combines over
+// the key ranges of a row.
+#pragma once
+#include "internal.h"
+#include "device_utils.cuh"
+#include "sm100_ptx.cuh"
+
+namespace attn {
+
+using namespace sm100;
+
+constexpr int BK = 64;                    // keys per chunk
+constexpr int SLOTS = 4;                  // ring slots, one chunk of K or V each
+constexpr int BUFS = 4;                   // S / P buffers in TMEM, 64 columns each: columns [0, 256)
+constexpr int TMEM_O = 256;               // O: columns [256, 256 + head_dim)
+constexpr int SUB_Q = 128 * 64 * 2;       // [128 rows][64 bf16] swizzled sub-tile of Q
+constexpr int SUB_KV = BK * 64 * 2;       // [64 keys][64 bf16] swizzled sub-tile of K or V
+constexpr float RESCALE = 8.f;            // log2 units a chunk's maximum may exceed the reference by
+
+__host__ __device__ constexpr int q_bytes(int dh) { return 2 * (dh / 64) * SUB_Q; }
+__host__ __device__ constexpr int slot_bytes(int dh) { return 2 * (dh / 64) * SUB_KV; }
+__host__ __device__ constexpr int smem_bytes(int dh) { return q_bytes(dh) + SLOTS * slot_bytes(dh); }
+
+struct Ctl {
+  unsigned long long full[SLOTS], empty[SLOTS];
+  unsigned long long q_full, q_empty;
+  unsigned long long s_full[BUFS], p_full[BUFS], pv_done[BUFS];
+  float red_max[2][2][128];               // [chunk parity][half of the chunk][row]
+  float red_sum[2][128];
+  int len[SPECASR_MAX_BATCH];             // committed length of every utterance, -1 if its tree was refused
+};
+
+__device__ __forceinline__ void ctl_init(Ctl* c) {
+  for (int s = 0; s < SLOTS; ++s) {
+    mbar_init(&c->full[s], 1);
+    mbar_init(&c->empty[s], 1);
+  }
+  mbar_init(&c->q_full, 1);
+  mbar_init(&c->q_empty, 1);
+  for (int b = 0; b < BUFS; ++b) {
+    mbar_init(&c->s_full[b], 1);
+    mbar_init(&c->p_full[b], 8);          // one arrival per soft-max warp
+    mbar_init(&c->pv_done[b], 1);
+  }
+}
+
+// The utterances' lengths and verdicts as all roles of the CTA are to see them (call before a barrier of the whole CTA).
+// They are read once: a status word can change while the kernel runs, when a bounded wait expires somewhere, and roles
+// that disagreed about which units to run would wait for one another in vain.
+__device__ __forceinline__ void snapshot(Ctl* c, const SegTable& tab) {
+  for (int b = threadIdx.x; b < tab.count; b += blockDim.x)
+    c->len[b] = *(volatile int32_t*)(tab.seg[b].ctl + CTL_STATUS) != 0 ? -1 : *(volatile int32_t*)(tab.seg[b].ctl + CTL_LEN);
+}
+
+// Unit `u` of a call: utterances in table order, each with splits x row tiles x KV heads units, heads fastest.
+struct Unit {
+  int seg, kvh, node0, split, k_begin;
+};
+__device__ __forceinline__ Unit unit_of(const SegTable& tab, int u, int Hkv, int nodes_per_tile) {
+  Unit r;
+  r.seg = 0;
+  while (r.seg + 1 < tab.count && u >= tab.seg[r.seg + 1].unit0) ++r.seg;
+  const SegDev& sg = tab.seg[r.seg];
+  u -= sg.unit0;
+  const int tiles = (sg.n + nodes_per_tile - 1) / nodes_per_tile;
+  const int rest = u / Hkv;
+  r.kvh = u - rest * Hkv;
+  r.split = rest / tiles;
+  r.node0 = (rest - r.split * tiles) * nodes_per_tile;
+  r.k_begin = r.split * sg.chunk;
+  return r;
+}
+
+// Whether the unit's utterance takes part, its length, and the unit's positions in use: 0 or fewer for a range beyond the
+// cache (the host knows only an upper bound of the length), which leaves an empty partial.
+__device__ __forceinline__ bool unit_live(const Ctl* c, const SegTable& tab, const Unit& un, int& L, int& kc) {
+  L = c->len[un.seg];
+  kc = min(tab.seg[un.seg].chunk, L + tab.seg[un.seg].n - un.k_begin);
+  return L >= 0;
+}
+
+// ---- TMA producer (one elected thread).  `pos` counts ring slots and `units` units since the kernel began.
+template <int DH, typename Wait>
+__device__ __forceinline__ bool produce(Ctl* c, uint8_t* smem, const CUtensorMap* tmQ, const SegDev& sg, int page_size,
+                                        int layer, const Unit& un, int kc, int group, int rows_used, int& pos, int& units,
+                                        Wait&& wait) {
+  constexpr int H = DH / 64;
+  const int n = (kc + BK - 1) / BK;
+  uint8_t* ring = smem + q_bytes(DH);
+  // the previous unit's score MMAs have read Q
+  if (!wait(&c->q_empty, (uint32_t)(units & 1) ^ 1u)) return false;
+  ++units;
+  mbar_expect_tx(&c->q_full, (uint32_t)(2 * H * rows_used * 128));
+#pragma unroll 1
+  for (int sub = 0; sub < 2 * H; ++sub)
+    tma_load_4d(smem + sub * SUB_Q, tmQ, (sub % H) * 64, un.kvh * group, sg.row0 + un.node0, sub / H, &c->q_full);
+#pragma unroll 1
+  for (int step = 0; step < 2 * n; ++step, ++pos) {     // K0, K1, V0, K2, V1, ..., V(n-1)
+    const bool is_v = step == 2 * n - 1 || (step >= 2 && (step & 1) == 0);
+    const int i = step == 0 ? 0 : is_v ? (step == 2 * n - 1 ? n - 1 : step / 2 - 1) : (step + 1) / 2;
+    const int keys = min(BK, kc - i * BK), groups = (keys + 15) >> 4;
+    const int slot = pos & (SLOTS - 1);
+    const int first = un.k_begin + i * BK;
+    int page[BK / 16], off[BK / 16];
+#pragma unroll
+    for (int g = 0; g < BK / 16; ++g) {                   // 16 keys never straddle a page
+      const int s = g < groups ? first + g * 16 : first;
+      page[g] = __ldg(sg.page_table + s / page_size);
+      off[g] = s % page_size;
+    }
+    if (!wait(&c->empty[slot], (uint32_t)((pos / SLOTS) & 1) ^ 1u)) return false;
+    mbar_expect_tx(&c->full[slot], (uint32_t)(2 * H * groups * 16 * 128));
+    uint8_t* dst = ring + slot * slot_bytes(DH);
+    const CUtensorMap* map = is_v ? sg.tmV : sg.tmK;
+#pragma unroll
+    for (int g = 0; g < BK / 16; ++g)
+      if (g < groups) {
+#pragma unroll
+        for (int sub = 0; sub < 2 * H; ++sub)
+          tma_load_5d(dst + sub * SUB_KV + g * 16 * 128, map, (sub % H) * 64, off[g], sub / H, un.kvh,
+                      layer * sg.n_pages + page[g], &c->full[slot]);
+      }
+  }
+  return true;
+}
+
+// ---- MMA issuer (one elected thread).  `g` counts chunks since the kernel began.
+template <int DH, typename Wait>
+__device__ __forceinline__ bool multiply(Ctl* c, uint8_t* smem, uint32_t tmem, int kc, int& pos, int& g, int& units,
+                                         Wait&& wait) {
+  constexpr int H = DH / 64;
+  const int n = (kc + BK - 1) / BK;
+  const uint32_t q_lo = smem_desc_lo(smem_u32(smem));
+  const uint32_t k_lo = smem_desc_lo(smem_u32(smem + q_bytes(DH)));
+  const uint32_t v_lo = smem_desc_lo(smem_u32(smem + q_bytes(DH)), SUB_KV);      // next 64 of head_dim: the next sub-tile
+  const uint32_t idesc_o = make_idesc_bf16(DH, true);
+  if (!wait(&c->q_full, (uint32_t)(units & 1))) return false;
+  ++units;
+#pragma unroll 1
+  for (int i = 0; i <= n; ++i) {
+    if (i < n) {                                            // scores of chunk i
+      const int slot = pos & (SLOTS - 1), b = (g + i) & (BUFS - 1), use = (g + i) / BUFS;
+      if (!wait(&c->full[slot], (uint32_t)((pos / SLOTS) & 1))) return false;
+      if (!wait(&c->pv_done[b], (uint32_t)(use & 1) ^ 1u)) return false;      // the buffer's last P has been read
+      tc_fence_after();
+      const int keys = min(BK, (kc - i * BK + 15) & ~15);
+      const uint32_t idesc_s = make_idesc_bf16(keys);
+      const uint32_t b_lo = k_lo + (uint32_t)((slot * slot_bytes(DH)) >> 4);
+      const uint32_t d = tmem + (uint32_t)(b * BK);
+#pragma unroll
+      for (int term = 0; term < 3; ++term) {               // hi*hi, hi*lo, lo*hi
+        const int qp = term == 2 ? 1 : 0, kp = term == 1 ? 1 : 0;
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            umma_bf16_lo(d, q_lo + (((qp * H + h) * SUB_Q + k * 32) >> 4), b_lo + (((kp * H + h) * SUB_KV + k * 32) >> 4),
+                         idesc_s, (term | h | k) ? 1u : 0u);
+        }
+      }
+      umma_commit(&c->s_full[b]);
+      umma_commit(&c->empty[slot]);
+      if (i == n - 1) umma_commit(&c->q_empty);
+      ++pos;
+    }
+    if (i > 0) {                                            // values of chunk i - 1
+      const int j = i - 1;
+      const int slot = pos & (SLOTS - 1), b = (g + j) & (BUFS - 1), use = (g + j) / BUFS;
+      if (!wait(&c->full[slot], (uint32_t)((pos / SLOTS) & 1))) return false;
+      if (!wait(&c->p_full[b], (uint32_t)(use & 1))) return false;
+      tc_fence_after();
+      const int steps = min(BK, (kc - j * BK + 15) & ~15) >> 4;
+      const uint32_t b_lo = v_lo + (uint32_t)((slot * slot_bytes(DH)) >> 4);
+      const uint32_t a = tmem + (uint32_t)(b * BK);
+      uint32_t acc = j > 0 ? 1u : 0u;
+#pragma unroll
+      for (int term = 0; term < 3; ++term) {
+        const int pp = term == 2 ? 1 : 0, vp = term == 1 ? 1 : 0;
+#pragma unroll
+        for (int k = 0; k < BK / 16; ++k)
+          if (k < steps) {
+            // P of 32 keys: 16 columns of hi words, then 16 of lo words
+            umma_bf16_ts(tmem + TMEM_O, a + (uint32_t)((k >> 1) * 32 + pp * 16 + (k & 1) * 8),
+                         b_lo + ((vp * H * SUB_KV + k * 2048) >> 4), idesc_o, acc);
+            acc = 1u;
+          }
+      }
+      umma_commit(&c->pv_done[b]);
+      umma_commit(&c->empty[slot]);
+      ++pos;
+    }
+  }
+  g += n;
+  return true;
+}
+
+// ---- soft-max and output (eight warps; warps w and w + 4 share a TMEM lane quadrant and a row's chunks: `half` 0 / 1).
+// Waits return a warp-uniform verdict.  `pos` and `g` as above, counted by every thread.
+struct RowState {
+  unsigned long long anc[4];              // ancestor-or-self bits of the row's node
+  bool valid;
+};
+__device__ __forceinline__ void pair_bar(int quad) { asm volatile("bar.sync %0, 64;" ::"r"(2 + quad) : "memory"); }
+
+// bit j = cache position base + j is visible to the row (committed prefix, or itself / an ancestor in the tree)
+__device__ __forceinline__ uint32_t visible_keys(const RowState& r, int base, int L) {
+  const int t0 = base - L;                      // tree slot of the first key
+  if (t0 <= -32) return 0xFFFFFFFFu;
+  const int ts = t0 > 0 ? t0 : 0;
+  uint32_t win = 0u;                            // ancestor bits of tree slots ts .. ts + 31
+  if (ts < SPECASR_MAX_NODES) {
+    const int w = ts >> 6, sh = ts & 63;
+    const unsigned long long a = w == 0 ? r.anc[0] : w == 1 ? r.anc[1] : w == 2 ? r.anc[2] : r.anc[3];
+    const unsigned long long b = w == 0 ? r.anc[1] : w == 1 ? r.anc[2] : w == 2 ? r.anc[3] : 0ull;
+    win = (uint32_t)(sh ? (a >> sh) | (b << (64 - sh)) : a);
+  }
+  return t0 < 0 ? ((1u << (-t0)) - 1u) | (win << (-t0)) : win;
+}
+
+template <int DH, typename Wait>
+__device__ __forceinline__ bool soften(Ctl* c, uint8_t* smem, uint32_t tmem, int kc, int k_begin, int L, float scale_log2,
+                                       const RowState& rs, int quad, int half, int& pos, int& g, float* out_row,
+                                       float2* out_ml, Wait&& wait) {
+  constexpr int H = DH / 64;
+  const int lane = threadIdx.x & 31;
+  const int row = quad * 32 + lane;
+  const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
+  const int n = (kc + BK - 1) / BK;
+  float m = -INFINITY, l = 0.f;
+  bool ok = true;
+#pragma unroll 1
+  for (int i = 0; i < n; ++i) {                            // no early exit: the pair's barriers must match
+    const int b = (g + i) & (BUFS - 1), use = (g + i) / BUFS;
+    if (ok) ok = wait(&c->s_full[b], (uint32_t)(use & 1));
+    tc_fence_after();
+    const uint32_t sp = tmem + lane_off + (uint32_t)(b * BK + half * 32);
+    const int k0 = i * BK + half * 32;                    // this thread's 32 keys within the unit's range
+    float s[32];
+    tmem_ld32(sp, s);                                      // after a failed wait: whatever is there, nothing uses it
+    uint32_t vis = 0u;
+    if (rs.valid && k0 < kc) {
+      vis = visible_keys(rs, k_begin + k0, L);
+      if (kc - k0 < 32) vis &= (1u << (kc - k0)) - 1u;
+    }
+    if (!__all_sync(0xFFFFFFFFu, vis == 0xFFFFFFFFu)) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) s[j] = ((vis >> j) & 1u) ? s[j] : -INFINITY;
+    }
+    float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+    for (int j = 0; j < 32; ++j) mx[j & 1] = fmaxf(mx[j & 1], s[j]);
+    c->red_max[i & 1][half][row] = fmaxf(mx[0], mx[1]) * scale_log2;
+    pair_bar(quad);
+    const float top = fmaxf(c->red_max[i & 1][0][row], c->red_max[i & 1][1][row]);
+    if (i == 0) {
+      m = top;
+    } else if (__any_sync(0xFFFFFFFFu, top > m + RESCALE)) {    // both warps of the pair come to the same verdict
+      const int pb = (g + i - 1) & (BUFS - 1), puse = (g + i - 1) / BUFS;
+      if (ok) ok = wait(&c->pv_done[pb], (uint32_t)(puse & 1));
+      tc_fence_after();
+      const bool up = top > m + RESCALE;                     // also the first visible key of a row (m = -inf)
+      const float f = up ? fast_exp2(m - top) : 1.f;
+      if (up) m = top;
+      l *= f;
+#pragma unroll 1
+      for (int c0 = half * 32; c0 < DH; c0 += 64) {
+        float o[32];
+        tmem_ld32(tmem + TMEM_O + lane_off + (uint32_t)c0, o);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) o[j] *= f;
+        tmem_st16(tmem + TMEM_O + lane_off + (uint32_t)c0, reinterpret_cast<const uint32_t*>(o));
+        tmem_st16(tmem + TMEM_O + lane_off + (uint32_t)(c0 + 16), reinterpret_cast<const uint32_t*>(o + 16));
+      }
+    }
+    const float ref = m > -INFINITY ? m : 0.f;               // a row that has seen nothing gives p = 0 everywhere
+    float sum[2] = {0.f, 0.f};
+    uint32_t hi[16], lo[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const float p0 = fast_exp2(fmaf(s[2 * j], scale_log2, -ref)), p1 = fast_exp2(fmaf(s[2 * j + 1], scale_log2, -ref));
+      sum[0] += p0;
+      sum[1] += p1;
+      split2_pack(p0, p1, hi[j], lo[j]);
+    }
+    l += sum[0] + sum[1];
+    tmem_st16(sp, hi);
+    tmem_st16(sp + 16, lo);
+    if (i == n - 1 && (kc & 15) != 0) {
+      // value rows past the end of the cache meet p = 0, but 0 * garbage could still be NaN: clear them
+      const int slot = (pos + 2 * n - 1) & (SLOTS - 1);
+      if (ok) ok = wait(&c->full[slot], (uint32_t)(((pos + 2 * n - 1) / SLOTS) & 1));
+      const int first = kc - i * BK;
+      if (ok && half == 0 && row < ((first + 15) & ~15) - first) {
+        uint8_t* v = smem + q_bytes(DH) + slot * slot_bytes(DH) + (first + row) * 128;
+#pragma unroll 1
+        for (int sub = 0; sub < 2 * H; ++sub)
+#pragma unroll 1
+          for (int e = 0; e < 8; ++e) *reinterpret_cast<uint4*>(v + sub * SUB_KV + e * 16) = make_uint4(0, 0, 0, 0);
+      }
+      fence_proxy_async_smem();
+    }
+    tmem_wait_st();
+    tc_fence_before();
+    __syncwarp();
+    if (ok && lane == 0) mbar_arrive(&c->p_full[b]);
+  }
+  c->red_sum[half][row] = l;
+  if (ok) {
+    const int b = (g + n - 1) & (BUFS - 1), use = (g + n - 1) / BUFS;
+    ok = wait(&c->pv_done[b], (uint32_t)(use & 1));
+  }
+  if (ok) {
+    tc_fence_after();
+#pragma unroll 1
+    for (int c0 = half * 32; c0 < DH; c0 += 64) {
+      float o[32];
+      tmem_ld32(tmem + TMEM_O + lane_off + (uint32_t)c0, o);
+      if (rs.valid) {
+        float4* dst = reinterpret_cast<float4*>(out_row + c0);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) dst[e] = make_float4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
+      }
+    }
+    tc_fence_before();
+  }
+  pair_bar(quad);                                           // both halves of every row's sum are in shared memory
+  if (ok && rs.valid && half == 0) *out_ml = make_float2(m, c->red_sum[0][row] + c->red_sum[1][row]);
+  pos += 2 * n;
+  g += n;
+  return ok;
+}
+
+}  // namespace attn

@@ -29,11 +29,9 @@
 // consumer of the projection multiplies by rsqrt(mean(x^2) + eps), which commutes with the projection.  That
 // removes the row-wide reduction from the path between two projections.
 //
-// The attention step borrows the ring's shared memory (Q / P tiles and K / V pages of one key block), so the
+// The attention step borrows the ring's shared memory (Q, and a ring of K / V chunks), so the
 // weight producer resumes when the CTA's attention units are done.
-#include "internal.h"
-#include "device_utils.cuh"
-#include "sm100_ptx.cuh"
+#include "attention_unit.cuh"
 
 using namespace sm100;
 
@@ -63,11 +61,6 @@ constexpr int WORKERS = 256;            // warps 2..9
 constexpr int NUM_THREADS = 352;        // + TMA weights, MMA, TMA activations
 constexpr int NORM_PARTS = 2;           // fixed halves of a row whose sums of squares are kept apart
 
-constexpr int KEYS_MAX = 208;           // cache positions per attention unit (13 pages of 16)
-constexpr int ROUND = 128;              // keys whose probabilities fit the P tile at once
-constexpr int SUB = 128 * 64 * 2;       // [128 rows][64 bf16] swizzled sub-tile (Q, P)
-constexpr int KVSUB = KEYS_MAX * 64 * 2;
-
 // steps of a layer, in order; step k of the call has its own arrival counter, complete when it equals the CTA count
 // (one shared counter would not do: a CTA without work in a step runs ahead and would be counted for a later one)
 enum { ST_NORM1 = 0, ST_QKV, ST_ROPE, ST_ATTN, ST_MERGE, ST_O, ST_NORM2, ST_GU, ST_DOWN, ST_PER_LAYER };
@@ -77,20 +70,16 @@ struct alignas(16) StackCtl {
   unsigned long long empty[MAX_STAGES];
   unsigned long long acc_full[2];
   unsigned long long acc_empty[2];
-  unsigned long long bar_qk, bar_v, bar_s, bar_p[2], bar_o[2];
+  attn::Ctl att;
   unsigned long long key[64];
   unsigned long long k1q[4][64], k2q[4][64];   // per lane quadrant: best and second-best packed key of a vocabulary tile
   float2 msq[4][64];                    // per lane quadrant: (max, sum of exp(x - max)) over the tile's rows
-  float red_max[2][128];
-  float red_sum[2][128];
   float inv[64];                        // 1 / rms of every token row, for the epilogue in progress
   float red[8];
-  int page[KEYS_MAX / 16];               // pool page (of the layer) of every page of the attention unit
   uint32_t tmem_base;
   int abort;
   int attn_done;                        // attention steps this CTA has finished (its ring memory is free again)
   int step_ok;                          // verdict of a wait that one worker made for all of them
-  int units_done;                       // attention units the workers have finished (their shared memory is free again)
 };
 
 struct StackParams {
@@ -100,7 +89,7 @@ struct StackParams {
   const float* const* gains;            // [2 * n_layers + 1]: attention / FFN norm per layer, then the final norm
   const float2* rope;
   int n, n_pad, n_alloc, stages, stage_bytes, ring_bytes;
-  int splits_qkv, splits_o, splits_down, epoch0, want_head, group, nodes_per_tile, row_tiles, attn_units;
+  int splits_qkv, splits_o, splits_down, epoch0, want_head, group, nodes_per_tile;
   int32_t* ctl;                         // control block whose status word ends the call
   int32_t* sync;                        // [steps of the call] arrival counters, zeroed before the launch
   float* X;
@@ -285,15 +274,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmAO,
         const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmQ,
         const __grid_constant__ SegTable tab, const StackParams p) {
-  constexpr int H2 = DH / 64;                           // 64-wide halves of a head
-  constexpr int A_BYTES = 4 * SUB;                      // Q planes, later two P planes of 128 keys
   extern __shared__ uint8_t smem_raw[];
   uint8_t* ring = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   StackCtl* sc = (StackCtl*)(ring + p.ring_bytes);
   bf16* epi_stage = (bf16*)(sc + 1);                    // SiLU * up output tile [2 planes][tokens][64]
-  uint8_t* As = ring;                                   // attention: overlays the ring
-  uint8_t* KVs = ring + A_BYTES;
-
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int G = gridDim.x, cta = blockIdx.x;
   const int n_pad = p.n_pad;
@@ -309,21 +293,17 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
     for (int b = 0; b < 2; ++b) {
       mbar_init(&sc->acc_full[b], 1);
       mbar_init(&sc->acc_empty[b], WORKERS);
-      mbar_init(&sc->bar_p[b], WORKERS);
-      mbar_init(&sc->bar_o[b], 1);
     }
-    mbar_init(&sc->bar_qk, 1);
-    mbar_init(&sc->bar_v, 1);
-    mbar_init(&sc->bar_s, 1);
+    attn::ctl_init(&sc->att);
     sc->abort = 0;
     sc->attn_done = 0;
-    sc->units_done = 0;
     mbar_fence_init();
     tma_prefetch_desc(&tmH);
     tma_prefetch_desc(&tmAO);
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmQ);
   }
+  attn::snapshot(&sc->att, tab);
   if (warp == 1) tmem_alloc(&sc->tmem_base, 512);
   tc_fence_before();
   __syncthreads();
@@ -334,8 +314,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
   const bool live = *(volatile int32_t*)status == 0;
   const int n_steps = p.n_layers * ST_PER_LAYER + (p.want_head ? 2 : 0);   // final norm and vocabulary projection last
 
-  // attention geometry shared by all roles
-  const int rows_used = p.nodes_per_tile * p.group;
+  auto attn_wait = [&](void* bar, uint32_t parity) -> bool { return bar_wait(bar, parity, abort, status); };
 
   if (!live) {
     // the call was refused before it started (shared status): nothing to do
@@ -422,7 +401,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
     int slot = 0;                                        // next ring slot
     uint32_t ring_par = 0u;                              // parity of the ring round in progress
     bool ok = true;
-    int au = 0;                                          // attention units this CTA has run
+    int at_pos = 0, at_units = 0;                        // attention: ring slots filled, units run
     auto stream_acts = [&](const Gemm& g, const CUtensorMap* tmAct, int ready_step) {
       if (g.u1 <= g.u0) return;
       if (elect_one()) {
@@ -460,71 +439,30 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
         const CUtensorMap* tmAct = gk == ST_O ? &tmAO : gk == ST_DOWN ? &tmA : &tmH;
         stream_acts(gemm_of(p, l, gk, cta, G), tmAct, sidx - 1);
       } else if (l < p.n_layers && st == ST_ATTN) {
-        // ---- attention units of this CTA: one thread issues every box.
-        // (Asking for the K pages of a key block inside the committed prefix before the rotary step has finished
-        // made S ready 1.6 us earlier and the step no shorter; it was taken out again.)
-        bool rope_seen = false;
-        for (int u = cta; u < p.attn_units && ok; u += G) {
-          const int kvh = u % p.Hkv, tile_y = (u / p.Hkv) % p.row_tiles, z = u / (p.Hkv * p.row_tiles);
-          const int split = z % tab.splits;
-          const SegDev& sg = tab.seg[z / tab.splits];
-          const int node0 = tile_y * p.nodes_per_tile;
-          if (node0 >= sg.n || sg.ctl[CTL_STATUS] != 0) continue;
-          const int L = sg.ctl[CTL_LEN];
-          const int Ltot = L + sg.n;
-          const int k_begin = split * sg.chunk;
-          if (k_begin >= Ltot) continue;
-          const int kc = min(sg.chunk, Ltot - k_begin);
-          const int pages = (kc + p.page_size - 1) / p.page_size;
-          const uint32_t par = (uint32_t)(au & 1);
-          ++au;
-          // A CTA that runs several units reuses the Q / P and K / V tiles and the barriers: the next unit's loads
-          // (and the arming of its barriers) wait until the workers have stored the previous unit's output.
-          if (elect_one()) {
+        if (elect_one()) {
+          bool rope_seen = false;
+          int L = 0, kc = 0;
+#pragma unroll 1
+          for (int u = cta; u < tab.units && ok; u += G) {
+            const attn::Unit un = attn::unit_of(tab, u, p.Hkv, p.nodes_per_tile);
+            if (!attn::unit_live(&sc->att, tab, un, L, kc) || kc <= 0) continue;
             if (!rope_seen) {
               ok = wait_word_ge(p.sync + sidx - 1, G, abort, status);
               fence_proxy_async_all();
+              rope_seen = true;
             }
-            if (ok) ok = wait_smem_ge(&sc->units_done, au - 1, abort, status);
+            if (ok)
+              ok = attn::produce<DH>(&sc->att, ring, &tmQ, tab.seg[un.seg], p.page_size, l, un, kc, p.group,
+                                     p.nodes_per_tile * p.group, at_pos, at_units, attn_wait);
           }
-          rope_seen = true;
-          ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
-          if (!ok) break;
-          if (lane < pages) sc->page[lane] = l * sg.n_pages + sg.page_table[split * (sg.chunk / p.page_size) + lane];
-          __syncwarp();
-          if (elect_one()) {
-            const uint32_t q_bytes = 2 * H2 * rows_used * 128;
-            const uint32_t kv_bytes = 2 * H2 * pages * p.page_size * 128;
-            mbar_expect_tx(&sc->bar_qk, q_bytes + kv_bytes);
-            mbar_expect_tx(&sc->bar_v, kv_bytes);
-            for (int plane = 0; plane < 2; ++plane)
-              for (int h = 0; h < H2; ++h)
-                tma_load_4d(As + (plane * H2 + h) * SUB, &tmQ, h * 64, kvh * p.group, sg.row0 + node0, plane, &sc->bar_qk);
-            const CUtensorMap* map = sg.tmK;
-            void* bar = &sc->bar_qk;
-#pragma unroll 1
-            for (int kv = 0; kv < 2 && ok; ++kv) {
-#pragma unroll 1
-              for (int j = 0; j < pages; ++j) {
-                const int c4 = sc->page[j];
-                uint8_t* dst = KVs + j * p.page_size * 128;
-#pragma unroll
-                for (int sub = 0; sub < 2 * H2; ++sub)
-                  tma_load_5d(dst + sub * KVSUB, map, (sub % H2) * 64, 0, sub / H2, kvh, c4, bar);
-              }
-              // V takes K's place once the S MMAs have read K
-              if (kv == 0) ok = bar_wait(&sc->bar_s, par, abort, status);
-              map = sg.tmV;
-              bar = &sc->bar_v;
-            }
-          }
-          ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
         }
+        ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
       }
     }
   } else if (warp == 1 && elect_one()) {
     // =========================================================== MMA issuer
-    int slot = 0, seg = 0, au = 0, au2 = 0;
+    int slot = 0, seg = 0;
+    int at_pos = 0, at_g = 0, at_units = 0;              // attention: ring slots read, chunks and units run
     uint32_t ring_par = 0u;
     bool ok = true;
     const uint32_t ring_lo = smem_desc_lo(smem_u32(ring)), stage_lo = (uint32_t)(p.stage_bytes >> 4);
@@ -576,66 +514,11 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
       if (gk != -2) {
         run_gemm(gemm_of(p, l, gk, cta, G));
       } else if (l < p.n_layers && st == ST_ATTN) {
-        // ---- attention units
-        for (int u = cta; u < p.attn_units && ok; u += G) {
-          const int tile_y = (u / p.Hkv) % p.row_tiles, z = u / (p.Hkv * p.row_tiles);
-          const int split = z % tab.splits;
-          const SegDev& sg = tab.seg[z / tab.splits];
-          if (tile_y * p.nodes_per_tile >= sg.n || sg.ctl[CTL_STATUS] != 0) continue;
-          const int Ltot = sg.ctl[CTL_LEN] + sg.n;
-          const int k_begin = split * sg.chunk;
-          if (k_begin >= Ltot) continue;
-          const int kc = min(sg.chunk, Ltot - k_begin);
-          const int kc_pad = (kc + 15) & ~15;
-          const int rounds = (kc_pad + ROUND - 1) / ROUND;
-          const uint32_t par = (uint32_t)(au & 1);
-          ++au;
-          const uint32_t tmem_s = tmem_base, tmem_o = tmem_base + 256;
-          ok = bar_wait(&sc->bar_qk, par, abort, status);
-          if (!ok) break;
-          tc_fence_after();
-          {
-            const uint32_t idesc_s = make_idesc_bf16(kc_pad);
-            const uint32_t a_lo = smem_desc_lo(smem_u32(As)), b_lo = smem_desc_lo(smem_u32(KVs));
-  #pragma unroll
-            for (int term = 0; term < 3; ++term) {       // straight-line: a few instructions per MMA
-              const int qp = term == 2 ? 1 : 0, kp = term == 1 ? 1 : 0;     // hi*hi, hi*lo, lo*hi
-  #pragma unroll
-              for (int h = 0; h < H2; ++h) {
-  #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                  umma_bf16_lo(tmem_s, a_lo + (((qp * H2 + h) * SUB + k * 32) >> 4),
-                               b_lo + (((kp * H2 + h) * KVSUB + k * 32) >> 4), idesc_s, (term | h | k) ? 1u : 0u);
-              }
-            }
-            umma_commit(&sc->bar_s);
-          }
-          ok = bar_wait(&sc->bar_v, par, abort, status);
-          const uint32_t idesc2 = make_idesc_bf16(DH, true);
-          uint32_t acc = 0u;
-          for (int rd = 0; rd < rounds && ok; ++rd) {
-            const uint32_t par_r = rd == 0 ? par : (uint32_t)(au2 & 1);
-            ok = bar_wait(&sc->bar_p[rd], par_r, abort, status);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t a_lo = smem_desc_lo(smem_u32(As));
-            const uint32_t b_lo = smem_desc_lo(smem_u32(KVs), KVSUB) + (uint32_t)((rd * (ROUND / 16) * 2048) >> 4);
-            const int j_end = min(kc_pad - rd * ROUND, ROUND) / 16;
-  #pragma unroll
-            for (int term = 0; term < 3; ++term) {
-              const int pp = term == 2 ? 1 : 0, vp = term == 1 ? 1 : 0;
-  #pragma unroll
-              for (int j = 0; j < ROUND / 16; ++j) {
-                if (j < j_end) {
-                  umma_bf16_lo(tmem_o, a_lo + (((pp * 2 + (j >> 2)) * SUB + (j & 3) * 32) >> 4),
-                               b_lo + ((vp * H2 * KVSUB + j * 2048) >> 4), idesc2, acc);
-                  acc = 1u;
-                }
-              }
-            }
-            umma_commit(&sc->bar_o[rd]);
-          }
-          if (rounds == 2) ++au2;
+        int L = 0, kc = 0;
+#pragma unroll 1
+        for (int u = cta; u < tab.units && ok; u += G) {
+          const attn::Unit un = attn::unit_of(tab, u, p.Hkv, p.nodes_per_tile);
+          if (attn::unit_live(&sc->att, tab, un, L, kc) && kc > 0) ok = attn::multiply<DH>(&sc->att, ring, tmem_base, kc, at_pos, at_g, at_units, attn_wait);
         }
       }
     }
@@ -646,10 +529,10 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
     const int quad = warp & 3;
     const int row = quad * 32 + lane;                   // TMEM lane = output row of a weight tile / query row
     const int c_first = (wwarp >> 2) * 16;              // projections: this warp's first 16-token block, stride 32
-    const int eg = wwarp >> 2;                          // attention: which 32-key chunks this thread takes
+    const int eg = wwarp >> 2;                          // attention: which half of a 64-key chunk this thread takes
     const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
     bool ok = true;
-    int seg = 0, au = 0, au2 = 0;
+    int seg = 0, at_pos = 0, at_g = 0;
     int arrived = 0;                                     // steps this CTA has signed off
     int cur_layer = 0;
     (void)cur_layer;
@@ -1083,155 +966,28 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
       }
     };
 
-    // ---------------- attention: softmax over one key block, unnormalised partial out
+    // ---------------- attention: soft-max and unnormalised partial output of this CTA's units
     auto attention_step = [&]() {
       const size_t rows_alloc = (size_t)p.n_alloc * p.Hq;
+      int L = 0, kc = 0;
 #pragma unroll 1
-      for (int u = cta; u < p.attn_units; u += G) {
-        const int kvh = u % p.Hkv, tile_y = (u / p.Hkv) % p.row_tiles, z = u / (p.Hkv * p.row_tiles);
-        const int split = z % tab.splits;
-        const SegDev& sg = tab.seg[z / tab.splits];
-        const int node0 = tile_y * p.nodes_per_tile;
-        if (node0 >= sg.n || sg.ctl[CTL_STATUS] != 0) continue;
-        const int L = sg.ctl[CTL_LEN];
-        const int Ltot = L + sg.n;
-        const int k_begin = split * sg.chunk;
-        const int node = node0 + row / p.group;
-        const bool row_valid = row < rows_used && node < sg.n;
-        const size_t out_row = (size_t)split * rows_alloc + (size_t)(sg.row0 + node) * p.Hq + kvh * p.group + row % p.group;
-        if (k_begin >= Ltot) {                           // key block beyond the cache: an empty partial
-          if (row_valid && eg == 0) p.attML[out_row] = make_float2(-INFINITY, 0.f);
+      for (int u = cta; u < tab.units; u += G) {
+        const attn::Unit un = attn::unit_of(tab, u, p.Hkv, p.nodes_per_tile);
+        if (!attn::unit_live(&sc->att, tab, un, L, kc)) continue;
+        const SegDev& sg = tab.seg[un.seg];
+        const int node = un.node0 + row / p.group;
+        attn::RowState rs;
+        rs.valid = row < p.nodes_per_tile * p.group && node < sg.n;
+        const size_t out = (size_t)un.split * rows_alloc + (size_t)(sg.row0 + node) * p.Hq + un.kvh * p.group + row % p.group;
+        if (kc <= 0) {
+          if (rs.valid && eg == 0) p.attML[out] = make_float2(-INFINITY, 0.f);
           continue;
         }
-        const int kc = min(sg.chunk, Ltot - k_begin);
-        const int kc_pad = (kc + 15) & ~15;
-        const int rounds = (kc_pad + ROUND - 1) / ROUND;
-        const uint32_t par = (uint32_t)(au & 1);
-        ++au;
-        const uint32_t par2 = (uint32_t)(au2 & 1);
-        if (rounds == 2) ++au2;
-        const uint32_t tmem_s = tmem_base, tmem_o = tmem_base + 256;
-        unsigned long long anc0 = 0ull, anc1 = 0ull, anc2 = 0ull, anc3 = 0ull;
-        if (row_valid) {
-          const unsigned long long* an = p.anc + (size_t)(sg.row0 + node) * 4;
-          anc0 = an[0]; anc1 = an[1]; anc2 = an[2]; anc3 = an[3];
-        }
-        auto visible_keys = [&](int base) -> uint32_t {
-          const int t0 = base - L;                      // tree slot of the chunk's first key
-          if (t0 <= -32) return 0xFFFFFFFFu;            // all 32 keys lie in the committed prefix
-          const int ts = t0 > 0 ? t0 : 0;
-          uint32_t win = 0u;                            // ancestor bits of tree slots ts .. ts + 31
-          if (ts < SPECASR_MAX_NODES) {
-            const int w = ts >> 6, sh = ts & 63;
-            const unsigned long long a = w == 0 ? anc0 : w == 1 ? anc1 : w == 2 ? anc2 : anc3;
-            const unsigned long long bq = w == 0 ? anc1 : w == 1 ? anc2 : w == 2 ? anc3 : 0ull;
-            win = (uint32_t)(sh ? (a >> sh) | (bq << (64 - sh)) : a);
-          }
-          return t0 < 0 ? ((1u << (-t0)) - 1u) | (win << (-t0)) : win;
-        };
-        // bit j = key (k_begin + c0 + j) belongs to this unit's block and is visible to this row (16 keys; c0 < kc)
-        auto visible16 = [&](int c0) -> uint32_t {
-          const uint32_t mine = kc - c0 >= 16 ? 0xFFFFu : (1u << (kc - c0)) - 1u;
-          return mine & visible_keys(k_begin + c0);
-        };
-        if (ok) ok = wwait(&sc->bar_s, par);
-        STACK_TRACE_POINT(1, cur_layer);
-        float m_row = -INFINITY;
-        if (ok) {
-          tc_fence_after();
-          float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll 1
-          for (int c0 = eg * 16; c0 < kc_pad; c0 += 32) {        // short rolled loops: this code runs once per layer
-            float s[16];
-            tmem_ld16(tmem_s + lane_off + c0, s);
-            const uint32_t vis = c0 < kc ? visible16(c0) : 0u;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) m4[j & 3] = fmaxf(m4[j & 3], ((vis >> j) & 1u) ? s[j] * p.scale_log2 : -INFINITY);
-          }
-          m_row = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-        }
-        sc->red_max[eg][row] = m_row;
-        STACK_TRACE_POINT(4, cur_layer);
-        worker_bar();
-        m_row = fmaxf(sc->red_max[0][row], sc->red_max[1][row]);
-        const float m_use = m_row > -INFINITY ? m_row : 0.f;      // a fully masked row gives p = 0 everywhere
-        float l2[2] = {0.f, 0.f};
-#pragma unroll 1
-        for (int rd = 0; rd < rounds && ok; ++rd) {
-          // the P tile holds 128 keys: the second round waits until the first round's MMAs have read it
-          if (rd > 0) ok = wwait(&sc->bar_o[0], par);
-          if (!ok) break;
-          STACK_TRACE_POINT(5 + rd, cur_layer);
-          const int c_end = min(kc_pad, (rd + 1) * ROUND);
-#pragma unroll 1
-          for (int c0 = rd * ROUND + eg * 16; c0 < c_end; c0 += 32) {
-            float s[16];
-            tmem_ld16(tmem_s + lane_off + c0, s);
-            const uint32_t vis = c0 < kc ? visible16(c0) : 0u;
-#pragma unroll
-            for (int j = 0; j < 16; ++j) s[j] = ((vis >> j) & 1u) ? fast_exp2(s[j] * p.scale_log2 - m_use) : 0.f;
-#pragma unroll
-            for (int gq = 0; gq < 2; ++gq) {
-              uint32_t hi[4], lo[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const int j = gq * 8 + 2 * e;
-                l2[e & 1] += s[j] + s[j + 1];
-                split2_pack(s[j], s[j + 1], hi[e], lo[e]);
-              }
-              const int c8 = ((c0 - rd * ROUND) >> 3) + gq;     // 8-key group within this round's 128 keys
-              const int off = (c8 >> 3) * SUB + row * 128 + (((c8 & 7) ^ (row & 7)) << 4);
-              *reinterpret_cast<uint4*>(As + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-              *reinterpret_cast<uint4*>(As + 2 * SUB + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-            }
-          }
-          STACK_TRACE_POINT(7 + rd, cur_layer);
-          if (rd == rounds - 1 && kc < kc_pad) {
-            // value rows past the end of the cache meet p = 0, but 0 * garbage could still be NaN: clear them
-            ok = wwait(&sc->bar_v, par);
-            if (ok && eg == 0 && row < kc_pad - kc) {
-#pragma unroll 1
-              for (int sub = 0; sub < 2 * H2; ++sub)
-#pragma unroll 1
-                for (int i = 0; i < 8; ++i)
-                  *reinterpret_cast<uint4*>(KVs + sub * KVSUB + (kc + row) * 128 + i * 16) = make_uint4(0, 0, 0, 0);
-            }
-          }
-          if (ok) {
-            fence_proxy_async_smem();
-            mbar_arrive(&sc->bar_p[rd]);
-          }
-        }
-        sc->red_sum[eg][row] = l2[0] + l2[1];
-        STACK_TRACE_POINT(2, cur_layer);
-        if (ok) ok = rounds == 2 ? wwait(&sc->bar_o[1], par2) : wwait(&sc->bar_o[0], par);
-        STACK_TRACE_POINT(3, cur_layer);
-        // Every thread holds 32 consecutive floats of its row per TMEM load and stores them straight to the partial
-        // output: 128 contiguous bytes per thread, whole sectors.  (Staging the tile in shared memory so that a warp
-        // writes whole rows cost two more barriers and a pass of index arithmetic, 3 us against 1.)
-        if (ok) {                                               // warp-uniform: the TMEM load is a warp-wide instruction
-          tc_fence_after();
-          float4* dst = reinterpret_cast<float4*>(p.attO + out_row * DH);
-#pragma unroll 1
-          for (int c0 = eg * 32; c0 < DH; c0 += 64) {
-            float o[32];
-            tmem_ld32(tmem_o + lane_off + c0, o);
-            if (row_valid) {
-#pragma unroll
-              for (int e = 0; e < 8; ++e) dst[(c0 >> 2) + e] = make_float4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
-            }
-          }
-        }
-        tc_fence_before();
-        STACK_TRACE_POINT(9, cur_layer);
-        worker_bar();                                           // both halves of every row's sum are in shared memory
-        if (ok && row_valid && eg == 0) p.attML[out_row] = make_float2(m_row, sc->red_sum[0][row] + sc->red_sum[1][row]);
-        STACK_TRACE_POINT(13, cur_layer);
-        worker_bar();                                           // the staging area and red_* are free again
-        if (wtid == 0) {
-          __threadfence_block();
-          *(volatile int*)&sc->units_done = au;                 // units this CTA has finished since the kernel began
-        }
+        for (int w = 0; w < 4; ++w) rs.anc[w] = rs.valid ? p.anc[(size_t)(sg.row0 + node) * 4 + w] : 0ull;
+        const bool good = attn::soften<DH>(&sc->att, ring, tmem_base, kc, un.k_begin, L, p.scale_log2, rs, quad, eg, at_pos,
+                                           at_g, p.attO + out * DH, p.attML + out, wwait);
+        ok = ok && good;
       }
     };
 
@@ -1239,12 +995,12 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
     auto merge_step = [&]() {
       const size_t rows_alloc = (size_t)p.n_alloc * p.Hq;
       const int rows_total = p.n * p.Hq;
-      const int n_splits = tab.splits;
       const size_t ao_plane = (size_t)p.n_alloc * p.q_dim;
       const int c = lane * 4;
 #pragma unroll 1
       for (int r = cta * 8 + wwarp; r < rows_total; r += G * 8) {
         bf16* out = p.AO + (size_t)r * DH + c;
+        const int n_splits = tab.seg[seg_of_row(tab, r / p.Hq)].splits;
         const float2 none = make_float2(-INFINITY, 0.f);
         const float2 ml0 = lane < n_splits ? __ldcg(p.attML + (size_t)lane * rows_alloc + r) : none;
         const float2 ml1 = lane + 32 < n_splits ? __ldcg(p.attML + (size_t)(lane + 32) * rows_alloc + r) : none;
@@ -1386,11 +1142,10 @@ cudaError_t launch_dh(const CUtensorMap& tmH, const CUtensorMap& tmAO, const CUt
 
 // Shapes the fused kernel covers: tensor-core attention (head_dim 64 / 128, pages of a multiple of 16 slots),
 // up to 64 token rows (one activation box, both planes in one MMA), key-block count within one counter lane pair.
-bool fused_stack_supported(const specasr_kv* wk, int n_total, bool att_tc, int splits) {
+bool fused_stack_supported(const specasr_kv* wk, int n_total, bool att_tc) {
   const specasr_model* m = wk->m;
   if (m->cfg.gemm_path != 0 || !att_tc || !wk->attn_tc || m->w_maps_dev == nullptr) return false;
   if (n_total < 1 || n_total > 64) return false;
-  if (splits > kMaxAttnSplits) return false;
   // every weight tile of a linear projection needs a CTA of its own
   const int groups_qkv = (m->qkv_dim + TM * TILE_M - 1) / (TM * TILE_M);
   const int groups_d = (m->cfg.d_model + TM * TILE_M - 1) / (TM * TILE_M);
@@ -1402,7 +1157,7 @@ size_t fused_stack_sync_bytes(const specasr_model* m) {
   return (((size_t)m->cfg.n_layers * ST_PER_LAYER + 2) * sizeof(int32_t) + 255) / 256 * 256;
 }
 
-bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int n_total, int n_max,
+bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int n_total,
                         const int32_t* ctl_shared, bool want_head, float* out_logits, bool want_top2, cudaStream_t s) {
   const specasr_model_config& c = m->cfg;
   int n_pad = 16;
@@ -1420,7 +1175,7 @@ bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, i
   p.n = n_total; p.n_pad = n_pad; p.n_alloc = wk->n_alloc;
   p.stage_bytes = W_STAGE_BYTES + KSUB * n_pad * 2 * SUB_K * 2;
   const int epi_bytes = 2 * n_pad * 64 * 2;
-  const int attn_bytes = 4 * SUB + 2 * (c.head_dim / 64) * KVSUB;
+  const int attn_bytes = attn::smem_bytes(c.head_dim);
   int stages = (SMEM_LIMIT - (int)sizeof(StackCtl) - epi_bytes - 1024) / p.stage_bytes;
   if (stages > MAX_STAGES) stages = MAX_STAGES;
   p.stages = stages;
@@ -1443,8 +1198,6 @@ bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, i
   p.want_head = want_head ? 1 : 0;
   p.group = c.n_heads / c.n_kv_heads;
   p.nodes_per_tile = 128 / p.group;
-  p.row_tiles = (n_max + p.nodes_per_tile - 1) / p.nodes_per_tile;
-  p.attn_units = c.n_kv_heads * p.row_tiles * tab.count * tab.splits;
   p.ctl = const_cast<int32_t*>(ctl_shared);
   p.sync = wk->ws.sync;
   p.X = wk->ws.X; p.P = wk->ws.P; p.fixP = wk->ws.fixP; p.fixFlag = wk->ws.fixFlag;

@@ -205,14 +205,16 @@ struct SegDev {
   int n_pages;
   int row0;                     // first workspace row
   int n;                        // rows
-  int chunk;                    // keys per attention CTA
+  int chunk;                    // cache positions per attention unit, a multiple of 16
+  int splits;                   // attention units a row's positions are cut into
+  int unit0;                    // first attention unit of the utterance
   int capacity;                 // positions the cache can hold
-  int pad;
 };
 struct SegTable {
   int count;
-  int splits;                   // grid depth of the attention launch per utterance (largest any of them needs)
-  int pad[2];
+  int splits;                   // largest `splits` of any utterance
+  int units;                    // attention units of the call
+  int pad;
   SegDev seg[SPECASR_MAX_BATCH];
 };
 
@@ -228,7 +230,7 @@ void launch_copy_embeds(specasr_kv* kv, const float* embeds, int n, cudaStream_t
 void launch_rmsnorm_split(specasr_kv* wk, const int32_t* ctl, const float* gain, int n, int n_pad, int n_partials,
                           cudaStream_t s);
 void launch_rope_append(specasr_kv* wk, const SegTable& t, int n_total, int layer, int n_partials, cudaStream_t s);
-void launch_attn_merge(specasr_kv* wk, const int32_t* ctl, int n, int n_pad, int n_splits, cudaStream_t s);
+void launch_attn_merge(specasr_kv* wk, const SegTable& t, const int32_t* ctl, int n, int n_pad, cudaStream_t s);
 void launch_accept(specasr_kv* wk, const SegTable& t, const int32_t* ctl_shared, const int32_t* tokens,
                    const int32_t* parent, int n_tiles, int32_t* out_argmax, int32_t* out_accept_len, int32_t* out_path,
                    int32_t* out_bonus, cudaStream_t s);
@@ -239,15 +241,14 @@ void launch_commit(specasr_kv* kv, const int32_t* path, const int32_t* accept_le
 // ---- attention.cu (plain FMA) / attention_tc.cu (tcgen05)
 void launch_tree_attention(specasr_kv* kv, int layer, int n, int n_splits, cudaStream_t s);
 bool attention_tc_supported(const specasr_model* m);
-bool attention_tc_plan(const specasr_model* m, int n, int total_len, int sm_budget, int max_splits, int* n_splits,
-                       int* chunk);
+void attention_tc_plan(const specasr_model* m, SegTable* tab, const int* len_upper);   // fills chunk, splits, unit0, units
 bool attention_tc_make_maps(specasr_kv* kv);
-void launch_tree_attention_tc(specasr_kv* wk, const SegTable& t, int n_max, int layer, cudaStream_t s);
+void launch_tree_attention_tc(specasr_kv* wk, const SegTable& t, int layer, cudaStream_t s);
 
 // ---- fused_stack.cu: the whole layer stack as one persistent kernel
-bool fused_stack_supported(const specasr_kv* wk, int n_total, bool att_tc, int splits);
+bool fused_stack_supported(const specasr_kv* wk, int n_total, bool att_tc);
 size_t fused_stack_sync_bytes(const specasr_model* m);
-bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int n_total, int n_max,
+bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int n_total,
                         const int32_t* ctl_shared, bool want_head, float* out_logits, bool want_top2, cudaStream_t s);
 // top2.cu: top-2 tokens and probabilities of every node from the per-tile pieces the vocabulary epilogue left
 void launch_top2_from_tiles(specasr_kv* wk, const SegTable& t, const int32_t* ctl_shared, int n_total, int n_tiles,

@@ -404,8 +404,9 @@ void launch_rope_append(specasr_kv* wk, const SegTable& t, int n_total, int laye
 // (max, sum) of splits s and s + 32, lane c the output columns 4c .. 4c + 3; the partial outputs of
 // six splits are requested together (more would cost the registers that let the blocks wait beside the attention
 // kernel in one wave).  Rows n..n_pad-1 are zeroed.
-__global__ void __launch_bounds__(128) k_attn_merge(const int32_t* __restrict__ ctl, const float* __restrict__ attO,
-                                                    const float2* __restrict__ attML, int n_splits, size_t rows_alloc,
+__global__ void __launch_bounds__(128) k_attn_merge(const __grid_constant__ SegTable tab, const int32_t* __restrict__ ctl,
+                                                    const float* __restrict__ attO,
+                                                    const float2* __restrict__ attML, size_t rows_alloc,
                                                     int Hq, int dh, int n, int rows_total, bf16* __restrict__ AO,
                                                     size_t plane_stride SPECASR_TRACE_PARAM) {
   grid_dep_launch();
@@ -425,6 +426,7 @@ __global__ void __launch_bounds__(128) k_attn_merge(const int32_t* __restrict__ 
     }
     return;
   }
+  const int n_splits = tab.seg[segment_of_row(tab, row / Hq)].splits;
   const float2 none = make_float2(-INFINITY, 0.f);
   const float2 ml0 = lane < n_splits ? __ldcg(attML + (size_t)lane * rows_alloc + row) : none;
   const float2 ml1 = lane + 32 < n_splits ? __ldcg(attML + (size_t)(lane + 32) * rows_alloc + row) : none;
@@ -476,11 +478,11 @@ __global__ void __launch_bounds__(128) k_attn_merge(const int32_t* __restrict__ 
   }
 }
 
-void launch_attn_merge(specasr_kv* kv, const int32_t* ctl, int n, int n_pad, int n_splits, cudaStream_t s) {
+void launch_attn_merge(specasr_kv* kv, const SegTable& t, const int32_t* ctl, int n, int n_pad, cudaStream_t s) {
   const specasr_model_config& c = kv->m->cfg;
   const int rows_total = n_pad * c.n_heads;
   LaunchScope scope(kv, SPECASR_KIND_ATTN_MERGE, s);
-  launch_pdl(k_attn_merge, dim3((rows_total + 3) / 4), dim3(128), 0, s, ctl, kv->ws.attO, kv->ws.attML, n_splits,
+  launch_pdl(k_attn_merge, dim3((rows_total + 3) / 4), dim3(128), 0, s, t, ctl, kv->ws.attO, kv->ws.attML,
              (size_t)kv->n_alloc * c.n_heads, c.n_heads, c.head_dim, n, rows_total, kv->ws.AO,
              (size_t)kv->n_alloc * kv->m->q_dim SPECASR_TRACE_ARG(kv));
 }
