@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) k_tree_attention_tc(const __g
         if (!attn::unit_live(&sc->a, tab, un, L, kc) || kc <= 0) continue;
         int32_t* status = tab.seg[un.seg].ctl + CTL_STATUS;
         auto wait = [&](void* bar, uint32_t parity) -> bool { return mbar_wait(bar, parity, abort, status); };
-        if (!attn::produce<DH>(&sc->a, smem, &tmQ, tab.seg[un.seg], p.page_size, p.layer, un, kc, p.group,
+        if (!attn::produce<DH>(&sc->a, smem, &tmQ, tab.seg[un.seg], p.page_size, p.layer, p.Hkv, un, kc, p.group,
                                p.nodes_per_tile * p.group, pos, units, wait))
           break;
       }
@@ -222,11 +222,12 @@ bool attention_tc_make_maps(specasr_kv* kv) {
     if (!make_tensor_map_nd(&kv->tm_Q, kv->ws.Q, 4, dims, strides, box)) return false;
   }
   const uint64_t ps = c.page_size;
-  uint64_t dims[5] = {dh, ps, 2, (uint64_t)c.n_kv_heads, (uint64_t)c.n_layers * kv->n_pages};
-  uint64_t strides[4] = {dh * 2, ps * dh * 2, 2 * ps * dh * 2, (uint64_t)c.n_kv_heads * 2 * ps * dh * 2};
-  uint32_t box[5] = {64, 16, 1, 1, 1};             // 16 slots of a page: any page size the library takes is a multiple
-  if (!make_tensor_map_nd(&kv->tm_K, kv->k_pool, 5, dims, strides, box) ||
-      !make_tensor_map_nd(&kv->tm_V, kv->v_pool, 5, dims, strides, box))
+  // pools: [layer and page and kv head][plane][slot][dh]; box = 64 of dh, 16 slots (any page size is a multiple), both planes
+  uint64_t dims[4] = {dh, ps, 2, (uint64_t)c.n_layers * kv->n_pages * c.n_kv_heads};
+  uint64_t strides[3] = {dh * 2, ps * dh * 2, 2 * ps * dh * 2};
+  uint32_t box[4] = {64, 16, 2, 1};
+  if (!make_tensor_map_nd(&kv->tm_K, kv->k_pool, 4, dims, strides, box) ||
+      !make_tensor_map_nd(&kv->tm_V, kv->v_pool, 4, dims, strides, box))
     return false;
   // the kernel reads the pool descriptors through the utterance table, i.e. from global memory
   cudaError_t e = cudaMemcpy(kv->ws.tmKV, &kv->tm_K, sizeof(CUtensorMap), cudaMemcpyHostToDevice);

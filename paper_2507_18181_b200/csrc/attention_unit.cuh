@@ -6,17 +6,20 @@
 //
 // A unit is one KV head, a tile of up to 128 query rows (row = node * group + head-in-group, so a whole query group
 // shares every K/V element that is staged) and a range of cache positions, walked in chunks of 64 keys:
-//   S = Q K^T      M = 128 rows, N = 64 keys, K = head_dim        (Q and K in shared memory, both K-major)
+//   S = Q K^T      M = 128 rows, N = 64 keys x 2 planes, K = head_dim     (Q and K in shared memory, both K-major)
 //   P = exp2(S * scale - m), masked                                 (two threads per row, fp32, from TMEM)
 //   O += P V       M = 128 rows, N = head_dim, K = 64 keys         (P in TMEM, V the MN-major B operand)
-// Q, P, K and V are all carried as two bf16 planes (value ~ hi + lo); each product is three MMAs
-// (hi*hi + hi*lo + lo*hi) into the same fp32 accumulator, which keeps ~16 significant bits.
+// Q, P, K and V are all carried as two bf16 planes (value ~ hi + lo), which keeps ~16 significant bits.  K and V come as
+// boxes of 16 slots with both planes behind one another, so the planes of K interleave along N: one MMA of N = 128 gives
+// q K_hi and q K_lo side by side (the soft-max adds them), once for each plane of Q.  O takes three terms, P_hi V_hi,
+// P_hi V_lo and P_lo V_hi.
 //
-// What bounds it: the tensor pipe, 24 score MMAs of 48 clocks (N = 64 is bound by the fetch of Q from shared memory) and
-// 12 value MMAs of 64 per chunk of head_dim 128, about 1 us per 128 x 64 block, as long as the soft-max keeps under it.
+// What bounds it: the tensor pipe, 16 score MMAs and 12 value MMAs of 64 clocks per chunk of head_dim 128, 0.95 us per
+// 128 x 64 block, as long as the loads (8 boxes a chunk; one thread issues a box in ~75 clocks) and the soft-max
+// (~1300 clocks a chunk) keep under it.
 // Hence the pipeline: chunks of K and V come through one ring in the order the MMAs want them (K0, K1, V0, K2, V1,
-// ...), the scores of chunk i + 1 are issued before the values of chunk i, and P takes the place of its own S in
-// TMEM -- each thread overwrites exactly the columns it has read -- so that no probability passes through shared memory.
+// ...), the scores of chunk i + 1 are issued before the values of chunk i, and P goes to the value MMAs through TMEM, so
+// that no probability passes through shared memory.
 // The running maximum is only a reference: it is raised, and O rescaled, when a chunk exceeds it by more than 2^8.
 // (Before, a unit was a single shot of at most 208 keys whose loads, scores, soft-max and values followed one another:
 // 82 us per layer at 256 rows on 2048 positions of the 7B shape, 44 here; 44 against 24 at 33 rows on 4096 positions, and
@@ -35,20 +38,22 @@ using namespace sm100;
 
 constexpr int BK = 64;                    // keys per chunk
 constexpr int SLOTS = 4;                  // ring slots, one chunk of K or V each
-constexpr int BUFS = 4;                   // S / P buffers in TMEM, 64 columns each: columns [0, 256)
-constexpr int TMEM_O = 256;               // O: columns [256, 256 + head_dim)
+constexpr int TMEM_S = 0;                 // S: two buffers of 128 columns (per 16 keys: 16 of q K_hi, 16 of q K_lo)
+constexpr int TMEM_O = 256;               // O: head_dim columns
+constexpr int TMEM_P = 384;               // P: two buffers of 64 columns (per 32 keys: 16 of hi words, 16 of lo words)
 constexpr int SUB_Q = 128 * 64 * 2;       // [128 rows][64 bf16] swizzled sub-tile of Q
-constexpr int SUB_KV = BK * 64 * 2;       // [64 keys][64 bf16] swizzled sub-tile of K or V
+constexpr int GROUP_KV = 2 * 16 * 128;    // [2 planes][16 keys][64 bf16]: one TMA box
+constexpr int SUB_KV = BK / 16 * GROUP_KV;   // one 64-wide part of the head of a chunk
 constexpr float RESCALE = 8.f;            // log2 units a chunk's maximum may exceed the reference by
 
 __host__ __device__ constexpr int q_bytes(int dh) { return 2 * (dh / 64) * SUB_Q; }
-__host__ __device__ constexpr int slot_bytes(int dh) { return 2 * (dh / 64) * SUB_KV; }
+__host__ __device__ constexpr int slot_bytes(int dh) { return dh / 64 * SUB_KV; }
 __host__ __device__ constexpr int smem_bytes(int dh) { return q_bytes(dh) + SLOTS * slot_bytes(dh); }
 
 struct Ctl {
   unsigned long long full[SLOTS], empty[SLOTS];
   unsigned long long q_full, q_empty;
-  unsigned long long s_full[BUFS], p_full[BUFS], pv_done[BUFS];
+  unsigned long long s_full[2], p_full[2], pv_done[2];
   float red_max[2][2][128];               // [chunk parity][half of the chunk][row]
   float red_sum[2][128];
   int len[SPECASR_MAX_BATCH];             // committed length of every utterance, -1 if its tree was refused
@@ -61,7 +66,7 @@ __device__ __forceinline__ void ctl_init(Ctl* c) {
   }
   mbar_init(&c->q_full, 1);
   mbar_init(&c->q_empty, 1);
-  for (int b = 0; b < BUFS; ++b) {
+  for (int b = 0; b < 2; ++b) {
     mbar_init(&c->s_full[b], 1);
     mbar_init(&c->p_full[b], 8);          // one arrival per soft-max warp
     mbar_init(&c->pv_done[b], 1);
@@ -106,7 +111,7 @@ __device__ __forceinline__ bool unit_live(const Ctl* c, const SegTable& tab, con
 // ---- TMA producer (one elected thread).  `pos` counts ring slots and `units` units since the kernel began.
 template <int DH, typename Wait>
 __device__ __forceinline__ bool produce(Ctl* c, uint8_t* smem, const CUtensorMap* tmQ, const SegDev& sg, int page_size,
-                                        int layer, const Unit& un, int kc, int group, int rows_used, int& pos, int& units,
+                                        int layer, int Hkv, const Unit& un, int kc, int group, int rows_used, int& pos, int& units,
                                         Wait&& wait) {
   constexpr int H = DH / 64;
   const int n = (kc + BK - 1) / BK;
@@ -140,9 +145,9 @@ __device__ __forceinline__ bool produce(Ctl* c, uint8_t* smem, const CUtensorMap
     for (int g = 0; g < BK / 16; ++g)
       if (g < groups) {
 #pragma unroll
-        for (int sub = 0; sub < 2 * H; ++sub)
-          tma_load_5d(dst + sub * SUB_KV + g * 16 * 128, map, (sub % H) * 64, off[g], sub / H, un.kvh,
-                      layer * sg.n_pages + page[g], &c->full[slot]);
+        for (int h = 0; h < H; ++h)
+          tma_load_4d(dst + h * SUB_KV + g * GROUP_KV, map, h * 64, off[g], 0, (layer * sg.n_pages + page[g]) * Hkv + un.kvh,
+                      &c->full[slot]);
       }
   }
   return true;
@@ -163,23 +168,21 @@ __device__ __forceinline__ bool multiply(Ctl* c, uint8_t* smem, uint32_t tmem, i
 #pragma unroll 1
   for (int i = 0; i <= n; ++i) {
     if (i < n) {                                            // scores of chunk i
-      const int slot = pos & (SLOTS - 1), b = (g + i) & (BUFS - 1), use = (g + i) / BUFS;
+      // its S buffer is free: the values of chunk i - 2, issued by this thread, waited for that chunk's soft-max
+      const int slot = pos & (SLOTS - 1), b = (g + i) & 1;
       if (!wait(&c->full[slot], (uint32_t)((pos / SLOTS) & 1))) return false;
-      if (!wait(&c->pv_done[b], (uint32_t)(use & 1) ^ 1u)) return false;      // the buffer's last P has been read
       tc_fence_after();
-      const int keys = min(BK, (kc - i * BK + 15) & ~15);
-      const uint32_t idesc_s = make_idesc_bf16(keys);
+      const uint32_t idesc_s = make_idesc_bf16(2 * min(BK, (kc - i * BK + 15) & ~15));
       const uint32_t b_lo = k_lo + (uint32_t)((slot * slot_bytes(DH)) >> 4);
-      const uint32_t d = tmem + (uint32_t)(b * BK);
+      const uint32_t d = tmem + (uint32_t)(TMEM_S + b * 2 * BK);
 #pragma unroll
-      for (int term = 0; term < 3; ++term) {               // hi*hi, hi*lo, lo*hi
-        const int qp = term == 2 ? 1 : 0, kp = term == 1 ? 1 : 0;
+      for (int qp = 0; qp < 2; ++qp) {
 #pragma unroll
         for (int h = 0; h < H; ++h) {
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            umma_bf16_lo(d, q_lo + (((qp * H + h) * SUB_Q + k * 32) >> 4), b_lo + (((kp * H + h) * SUB_KV + k * 32) >> 4),
-                         idesc_s, (term | h | k) ? 1u : 0u);
+            umma_bf16_lo(d, q_lo + (((qp * H + h) * SUB_Q + k * 32) >> 4), b_lo + ((h * SUB_KV + k * 32) >> 4), idesc_s,
+                         (qp | h | k) ? 1u : 0u);
         }
       }
       umma_commit(&c->s_full[b]);
@@ -189,13 +192,13 @@ __device__ __forceinline__ bool multiply(Ctl* c, uint8_t* smem, uint32_t tmem, i
     }
     if (i > 0) {                                            // values of chunk i - 1
       const int j = i - 1;
-      const int slot = pos & (SLOTS - 1), b = (g + j) & (BUFS - 1), use = (g + j) / BUFS;
+      const int slot = pos & (SLOTS - 1), b = (g + j) & 1, use = (g + j) >> 1;
       if (!wait(&c->full[slot], (uint32_t)((pos / SLOTS) & 1))) return false;
       if (!wait(&c->p_full[b], (uint32_t)(use & 1))) return false;
       tc_fence_after();
       const int steps = min(BK, (kc - j * BK + 15) & ~15) >> 4;
       const uint32_t b_lo = v_lo + (uint32_t)((slot * slot_bytes(DH)) >> 4);
-      const uint32_t a = tmem + (uint32_t)(b * BK);
+      const uint32_t a = tmem + (uint32_t)(TMEM_P + b * BK);
       uint32_t acc = j > 0 ? 1u : 0u;
 #pragma unroll
       for (int term = 0; term < 3; ++term) {
@@ -205,7 +208,7 @@ __device__ __forceinline__ bool multiply(Ctl* c, uint8_t* smem, uint32_t tmem, i
           if (k < steps) {
             // P of 32 keys: 16 columns of hi words, then 16 of lo words
             umma_bf16_ts(tmem + TMEM_O, a + (uint32_t)((k >> 1) * 32 + pp * 16 + (k & 1) * 8),
-                         b_lo + ((vp * H * SUB_KV + k * 2048) >> 4), idesc_o, acc);
+                         b_lo + ((k * GROUP_KV + vp * (GROUP_KV / 2)) >> 4), idesc_o, acc);
             acc = 1u;
           }
       }
@@ -254,13 +257,19 @@ __device__ __forceinline__ bool soften(Ctl* c, uint8_t* smem, uint32_t tmem, int
   bool ok = true;
 #pragma unroll 1
   for (int i = 0; i < n; ++i) {                            // no early exit: the pair's barriers must match
-    const int b = (g + i) & (BUFS - 1), use = (g + i) / BUFS;
+    const int b = (g + i) & 1, use = (g + i) >> 1;
+    // the scores of this chunk are complete, and with them the values of chunk i - 2: its P buffer is free too
     if (ok) ok = wait(&c->s_full[b], (uint32_t)(use & 1));
     tc_fence_after();
-    const uint32_t sp = tmem + lane_off + (uint32_t)(b * BK + half * 32);
     const int k0 = i * BK + half * 32;                    // this thread's 32 keys within the unit's range
-    float s[32];
-    tmem_ld32(sp, s);                                      // after a failed wait: whatever is there, nothing uses it
+    float s[32];                                           // after a failed wait: whatever is there, nothing uses it
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      float both[32];
+      tmem_ld32(tmem + lane_off + (uint32_t)(TMEM_S + b * 2 * BK + half * 64 + q * 32), both);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) s[q * 16 + j] = both[j] + both[16 + j];
+    }
     uint32_t vis = 0u;
     if (rs.valid && k0 < kc) {
       vis = visible_keys(rs, k_begin + k0, L);
@@ -279,7 +288,7 @@ __device__ __forceinline__ bool soften(Ctl* c, uint8_t* smem, uint32_t tmem, int
     if (i == 0) {
       m = top;
     } else if (__any_sync(0xFFFFFFFFu, top > m + RESCALE)) {    // both warps of the pair come to the same verdict
-      const int pb = (g + i - 1) & (BUFS - 1), puse = (g + i - 1) / BUFS;
+      const int pb = (g + i - 1) & 1, puse = (g + i - 1) >> 1;
       if (ok) ok = wait(&c->pv_done[pb], (uint32_t)(puse & 1));
       tc_fence_after();
       const bool up = top > m + RESCALE;                     // also the first visible key of a row (m = -inf)
@@ -307,6 +316,7 @@ __device__ __forceinline__ bool soften(Ctl* c, uint8_t* smem, uint32_t tmem, int
       split2_pack(p0, p1, hi[j], lo[j]);
     }
     l += sum[0] + sum[1];
+    const uint32_t sp = tmem + lane_off + (uint32_t)(TMEM_P + b * BK + half * 32);
     tmem_st16(sp, hi);
     tmem_st16(sp + 16, lo);
     if (i == n - 1 && (kc & 15) != 0) {
@@ -315,11 +325,13 @@ __device__ __forceinline__ bool soften(Ctl* c, uint8_t* smem, uint32_t tmem, int
       if (ok) ok = wait(&c->full[slot], (uint32_t)(((pos + 2 * n - 1) / SLOTS) & 1));
       const int first = kc - i * BK;
       if (ok && half == 0 && row < ((first + 15) & ~15) - first) {
-        uint8_t* v = smem + q_bytes(DH) + slot * slot_bytes(DH) + (first + row) * 128;
+        const int key = first + row;
+        uint8_t* v = smem + q_bytes(DH) + slot * slot_bytes(DH) + (key >> 4) * GROUP_KV + (key & 15) * 128;
 #pragma unroll 1
-        for (int sub = 0; sub < 2 * H; ++sub)
+        for (int sub = 0; sub < 2 * H; ++sub)              // planes of each 64-wide part of the head
 #pragma unroll 1
-          for (int e = 0; e < 8; ++e) *reinterpret_cast<uint4*>(v + sub * SUB_KV + e * 16) = make_uint4(0, 0, 0, 0);
+          for (int e = 0; e < 8; ++e)
+            *reinterpret_cast<uint4*>(v + (sub >> 1) * SUB_KV + (sub & 1) * (GROUP_KV / 2) + e * 16) = make_uint4(0, 0, 0, 0);
       }
       fence_proxy_async_smem();
     }
@@ -330,7 +342,7 @@ __device__ __forceinline__ bool soften(Ctl* c, uint8_t* smem, uint32_t tmem, int
   }
   c->red_sum[half][row] = l;
   if (ok) {
-    const int b = (g + n - 1) & (BUFS - 1), use = (g + n - 1) / BUFS;
+    const int b = (g + n - 1) & 1, use = (g + n - 1) >> 1;
     ok = wait(&c->pv_done[b], (uint32_t)(use & 1));
   }
   if (ok) {

@@ -452,7 +452,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
               rope_seen = true;
             }
             if (ok)
-              ok = attn::produce<DH>(&sc->att, ring, &tmQ, tab.seg[un.seg], p.page_size, l, un, kc, p.group,
+              ok = attn::produce<DH>(&sc->att, ring, &tmQ, tab.seg[un.seg], p.page_size, l, p.Hkv, un, kc, p.group,
                                      p.nodes_per_tile * p.group, at_pos, at_units, attn_wait);
           }
         }
