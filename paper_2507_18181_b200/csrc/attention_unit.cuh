@@ -123,19 +123,27 @@ __device__ __forceinline__ bool produce(Ctl* c, uint8_t* smem, const CUtensorMap
 #pragma unroll 1
   for (int sub = 0; sub < 2 * H; ++sub)
     tma_load_4d(smem + sub * SUB_Q, tmQ, (sub % H) * 64, un.kvh * group, sg.row0 + un.node0, sub / H, &c->q_full);
+  // page-table index and offset in the page of the next 16 keys of K and of V
+  int k_page = un.k_begin / page_size, k_off = un.k_begin - k_page * page_size;
+  int v_page = k_page, v_off = k_off;
 #pragma unroll 1
   for (int step = 0; step < 2 * n; ++step, ++pos) {     // K0, K1, V0, K2, V1, ..., V(n-1)
     const bool is_v = step == 2 * n - 1 || (step >= 2 && (step & 1) == 0);
     const int i = step == 0 ? 0 : is_v ? (step == 2 * n - 1 ? n - 1 : step / 2 - 1) : (step + 1) / 2;
     const int keys = min(BK, kc - i * BK), groups = (keys + 15) >> 4;
     const int slot = pos & (SLOTS - 1);
-    const int first = un.k_begin + i * BK;
+    int& idx = is_v ? v_page : k_page;
+    int& at = is_v ? v_off : k_off;
     int page[BK / 16], off[BK / 16];
 #pragma unroll
     for (int g = 0; g < BK / 16; ++g) {                   // 16 keys never straddle a page
-      const int s = g < groups ? first + g * 16 : first;
-      page[g] = __ldg(sg.page_table + s / page_size);
-      off[g] = s % page_size;
+      off[g] = at;
+      page[g] = g < groups ? __ldg(sg.page_table + idx) : 0;
+      at += 16;
+      if (at == page_size) {
+        at = 0;
+        ++idx;
+      }
     }
     if (!wait(&c->empty[slot], (uint32_t)((pos / SLOTS) & 1) ^ 1u)) return false;
     mbar_expect_tx(&c->full[slot], (uint32_t)(2 * H * groups * 16 * 128));

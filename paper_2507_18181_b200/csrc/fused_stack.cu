@@ -182,12 +182,19 @@ __device__ __forceinline__ int gemm_kind_of(int l, int st, int n_layers) {
 }
 
 // The polling loops are kept out of line: the kernel has some forty waits, and its text is fetched again on every
-// layer, so a copy of the loop at each of them is paid for in instruction-cache misses.
-__device__ __noinline__ bool bar_wait(void* bar, uint32_t parity, volatile int* abort, int32_t* status) {
+// layer, so a copy of the loop at each of them is paid for in instruction-cache misses.  The first try is in line: most
+// waits find their barrier complete, and the call alone cost about 450 clocks (90 in line).
+__device__ __noinline__ bool bar_poll(void* bar, uint32_t parity, volatile int* abort, int32_t* status) {
   return mbar_wait(bar, parity, abort, status);
 }
-__device__ __noinline__ bool bar_wait_relaxed(void* bar, uint32_t parity, volatile int* abort, int32_t* status) {
+__device__ __noinline__ bool bar_poll_relaxed(void* bar, uint32_t parity, volatile int* abort, int32_t* status) {
   return mbar_wait_relaxed(bar, parity, abort, status);
+}
+__device__ __forceinline__ bool bar_wait(void* bar, uint32_t parity, volatile int* abort, int32_t* status) {
+  return mbar_try(bar, parity) || bar_poll(bar, parity, abort, status);
+}
+__device__ __forceinline__ bool bar_wait_relaxed(void* bar, uint32_t parity, volatile int* abort, int32_t* status) {
+  return mbar_try(bar, parity) || bar_poll_relaxed(bar, parity, abort, status);
 }
 
 // Bounded poll of a word that only grows.  Returns false when the limit ran out or the call was aborted.
