@@ -122,8 +122,9 @@ __device__ __forceinline__ int ld_acquire(const int32_t* p) {
 __device__ __forceinline__ void st_release(int32_t* p, int v) {
   asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-__device__ __forceinline__ void red_release_add(int32_t* p, int v) {
-  asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+__device__ __forceinline__ void red_relaxed_add(int32_t* p, int v) {
+  asm volatile("red.relaxed.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 // generic-proxy accesses (ordinary loads / stores) <-> async-proxy accesses (TMA) of the same memory
 __device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
@@ -187,14 +188,8 @@ __device__ __forceinline__ int gemm_kind_of(int l, int st, int n_layers) {
 __device__ __noinline__ bool bar_poll(void* bar, uint32_t parity, volatile int* abort, int32_t* status) {
   return mbar_wait(bar, parity, abort, status);
 }
-__device__ __noinline__ bool bar_poll_relaxed(void* bar, uint32_t parity, volatile int* abort, int32_t* status) {
-  return mbar_wait_relaxed(bar, parity, abort, status);
-}
 __device__ __forceinline__ bool bar_wait(void* bar, uint32_t parity, volatile int* abort, int32_t* status) {
   return mbar_try(bar, parity) || bar_poll(bar, parity, abort, status);
-}
-__device__ __forceinline__ bool bar_wait_relaxed(void* bar, uint32_t parity, volatile int* abort, int32_t* status) {
-  return mbar_try(bar, parity) || bar_poll_relaxed(bar, parity, abort, status);
 }
 
 // Bounded poll of a word that only grows.  Returns false when the limit ran out or the call was aborted.
@@ -550,16 +545,13 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
     auto wwait = [&](void* bar, uint32_t parity) -> bool {
       return __all_sync(0xFFFFFFFFu, bar_wait(bar, parity, abort, status) ? 1 : 0) != 0;
     };
-    auto wwait_relaxed = [&](void* bar, uint32_t parity) -> bool {
-      return __all_sync(0xFFFFFFFFu, bar_wait_relaxed(bar, parity, abort, status) ? 1 : 0) != 0;
-    };
     // every worker's global writes of the step are done and visible -> one arrival for the CTA
     auto arrive_step = [&]() {
       worker_bar();                                      // every worker's stores of the step are issued ...
       if (wtid == 0) {
-        __threadfence();                                 // ... and ordered before the arrival (cumulative over the barrier)
+        fence_acq_rel_gpu();                             // ... and ordered before the arrival (cumulative over the barrier)
         fence_proxy_async_global();                      // the next step may read them through TMA
-        red_release_add(p.sync + arrived, 1);
+        red_relaxed_add(p.sync + arrived, 1);            // release by the fence above: a second one would be paid again
       }
       ++arrived;
     };
@@ -668,7 +660,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
         const int kb1 = (g.u1 - u) < (g.KB - kb0) ? kb0 + (g.u1 - u) : g.KB;
         u += kb1 - kb0;
         const int b = seg & 1;
-        if (ok) ok = wwait_relaxed(&sc->acc_full[b], (uint32_t)((seg >> 1) & 1));
+        if (ok) ok = wwait(&sc->acc_full[b], (uint32_t)((seg >> 1) & 1));
         STACK_TRACE_POINT(10, cur_layer);
         tc_fence_after();
         if (!ok) continue;
@@ -726,7 +718,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
           worker_bar();
           ok = ok && sc->step_ok != 0;
         }
-        if (ok) ok = wwait_relaxed(&sc->acc_full[b], (uint32_t)((seg >> 1) & 1));
+        if (ok) ok = wwait(&sc->acc_full[b], (uint32_t)((seg >> 1) & 1));
         STACK_TRACE_POINT(kb0 != 0 ? 12 : 11, cur_layer);
         tc_fence_after();
         const uint32_t lane_base = tmem_base + lane_off + (uint32_t)(b * TM * acc_cols);
