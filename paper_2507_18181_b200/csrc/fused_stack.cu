@@ -31,6 +31,8 @@
 //
 // The attention step borrows the ring's shared memory (Q, and a ring of K / V chunks), so the
 // weight producer resumes when the CTA's attention units are done.
+#include <algorithm>
+
 #include "attention_unit.cuh"
 
 using namespace sm100;
@@ -89,7 +91,7 @@ struct StackParams {
   const float* const* gains;            // [2 * n_layers + 1]: attention / FFN norm per layer, then the final norm
   const float2* rope;
   int n, n_pad, n_alloc, stages, stage_bytes, ring_bytes;
-  int splits_qkv, splits_o, splits_down, epoch0, want_head, group, nodes_per_tile;
+  int splits_qkv, splits_o, splits_down, epoch0, want_head, group, nodes_per_tile, whole_gu, whole_lm;
   int32_t* ctl;                         // control block whose status word ends the call
   int32_t* sync;                        // [steps of the call] arrival counters, zeroed before the launch
   float* X;
@@ -136,17 +138,18 @@ struct Gemm {
   const CUtensorMap* tmW;
   int M, K, KB, Kt, tiles, groups, splits;   // tiles of 128 rows in groups of TM; splits > 0: linear output in `splits` k-parts per group
   int g_eff;                            // CTAs that take part
-  int U, u0, u1;                        // all (tile group, k-block) units; this CTA's range
+  int U, u0, u1;                        // all (tile group, k-block) units; this CTA's range (whole: no tile is split)
 };
 
 __device__ __forceinline__ Gemm gemm_of(const StackParams& p, int layer, int which, int cta, int G) {
   Gemm g;
+  int whole = 0;
   switch (which) {
     case ST_QKV: g.M = p.qkv_dim; g.K = p.d; g.splits = p.splits_qkv; g.tmW = p.w_maps + 4 * layer; break;
     case ST_O: g.M = p.d; g.K = p.q_dim; g.splits = p.splits_o; g.tmW = p.w_maps + 4 * layer + 1; break;
-    case ST_GU: g.M = 2 * p.ffn; g.K = p.d; g.splits = 0; g.tmW = p.w_maps + 4 * layer + 2; break;
+    case ST_GU: g.M = 2 * p.ffn; g.K = p.d; g.splits = 0; whole = p.whole_gu; g.tmW = p.w_maps + 4 * layer + 2; break;
     case ST_DOWN: g.M = p.d; g.K = p.ffn; g.splits = p.splits_down; g.tmW = p.w_maps + 4 * layer + 3; break;
-    default: g.M = p.vocab; g.K = p.d; g.splits = 0; g.tmW = p.w_maps + 4 * p.n_layers; break;      // vocabulary
+    default: g.M = p.vocab; g.K = p.d; g.splits = 0; whole = p.whole_lm; g.tmW = p.w_maps + 4 * p.n_layers; break;      // vocabulary
   }
   g.KB = (g.K + KSUB * SUB_K - 1) / (KSUB * SUB_K);
   g.Kt = packed_col_tiles(g.K);
@@ -159,6 +162,14 @@ __device__ __forceinline__ Gemm gemm_of(const StackParams& p, int layer, int whi
       const int tile = cta / g.splits, split = cta % g.splits;
       g.u0 = tile * g.KB + split * g.KB / g.splits;
       g.u1 = tile * g.KB + (split + 1) * g.KB / g.splits;
+    } else {
+      g.u0 = g.u1 = 0;
+    }
+  } else if (whole) {
+    g.g_eff = g.groups < G ? g.groups : G;
+    if (cta < g.g_eff) {
+      g.u0 = cta * g.groups / g.g_eff * g.KB;
+      g.u1 = (cta + 1) * g.groups / g.g_eff * g.KB;
     } else {
       g.u0 = g.u1 = 0;
     }
@@ -740,10 +751,9 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
             }
             tc_fence_before();
             mbar_arrive(&sc->acc_empty[b]);
-            __threadfence();
           }
           worker_bar();
-          if (ok && wtid == 0) st_release(p.fixFlag + cta, epoch);
+          if (ok && wtid == 0) st_release(p.fixFlag + cta, epoch);     // a release is cumulative over the barrier
           continue;
         }
 
@@ -1192,6 +1202,20 @@ bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, i
   p.splits_qkv = pick_splits(m->qkv_dim, c.d_model);
   p.splits_o = pick_splits(c.d_model, m->q_dim);
   p.splits_down = pick_splits(c.d_model, c.ffn);
+  // Gate/up and vocabulary projections: whole tiles per CTA, or equal unit ranges with split tiles completed through
+  // parked partials.  Equal ranges keep every SM streaming to the end but pay for the fix-up (kFixupUs); whole tiles leave
+  // SMs idle in the last round, in which the others may still use the whole bandwidth up to what one SM can take in.
+  auto whole_tiles = [&](int M, int K) {
+    const double kFixupUs = 4.0, kHbm = 7.0e6, kIngest = 15.0e6, kSm = 0.103e6;      // bytes per us
+    const int G = m->n_sm, tiles = (M + TILE_M - 1) / TILE_M, KB = (K + KSUB * SUB_K - 1) / (KSUB * SUB_K);
+    const double all = std::max(W_STAGE_BYTES * G / kHbm, p.stage_bytes * G / kIngest), one = p.stage_bytes / kSm;
+    const int rounds = (tiles - 1) / G, rest = tiles - rounds * G;
+    const double whole = KB * (rounds * std::max(all, one) + std::max(one, all * rest / G));
+    const double ranges = std::max(all * tiles * KB / G, one) + kFixupUs;
+    return whole < ranges ? 1 : 0;
+  };
+  p.whole_gu = whole_tiles(2 * c.ffn, c.d_model);
+  p.whole_lm = whole_tiles(c.vocab, c.d_model);
   p.epoch0 = wk->gemm_epoch;
   wk->gemm_epoch += c.n_layers + 1;
   p.want_head = want_head ? 1 : 0;

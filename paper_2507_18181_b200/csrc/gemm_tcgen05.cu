@@ -336,10 +336,9 @@ __global__ void __launch_bounds__(64 + EPI_THREADS, 1) k_proj(const __grid_const
             for (int j = 0; j < 16; ++j) dst[(size_t)(c0 + j) * TILE_M + row] = v[j];
           }
           release_acc(b);
-          __threadfence();
         }
         epi_bar();
-        if (ok && etid == 0) st_release(p.fixFlag + cta, p.epoch);
+        if (ok && etid == 0) st_release(p.fixFlag + cta, p.epoch);       // a release is cumulative over the barrier
         continue;
       }
 
