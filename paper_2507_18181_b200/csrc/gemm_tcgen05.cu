@@ -192,6 +192,16 @@ __global__ void __launch_bounds__(64 + EPI_THREADS, 1) k_proj(const __grid_const
           par ^= 1u;
         }
       }
+      // The leader's commits arrive on both CTAs.  Those of the last stages, which nothing else waits for, have to land
+      // before this CTA leaves: its shared memory then belongs to another kernel, whose barriers they would hit.
+      if (total < p.stages) s = 0;
+      for (int i = 0; i < pre; ++i) {
+        if (!mbar_wait(&sc->empty[s], par, abort, status)) break;
+        if (++s == p.stages) {
+          s = 0;
+          par ^= 1u;
+        }
+      }
     }
   } else if (warp == 1 && rank == 0 && elect_one()) {
     // ---------------- MMA issuer of the pair
