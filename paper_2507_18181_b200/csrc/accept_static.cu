@@ -14,7 +14,7 @@
 
 namespace {
 
-constexpr int kStaticChunks = 64;                                     // vocabulary slices per node
+constexpr int kStaticChunks = 64;                                     // vocabulary slices per node, at most
 constexpr int kStaticCtlBytes = 256;                                  // word 0: device status of the last call
 constexpr size_t kStaticKeyBytes = (size_t)kStaticChunks * SPECASR_MAX_NODES * sizeof(unsigned long long);
 constexpr size_t kStaticBytes = kStaticCtlBytes + kStaticKeyBytes;    // 131328 bytes held by every device that loads the library
@@ -27,14 +27,22 @@ constexpr int kMaxDevices = 64;
 std::mutex g_static_mutex;
 void* g_static_ptr[kMaxDevices];     // device address of g_static_scratch, per device, filled on first use
 
-__global__ void __launch_bounds__(256) k_logit_keys_static(const float* __restrict__ logits, int vocab, int n,
+// Arg-max of one slice of one row's vocabulary.  Bound by the stream of the logits; the host picks the number of slices
+// so that rows x slices fill the GPU about four times (64 rows of 32000: 10 slices, 640 blocks of 13 values per thread;
+// 64 slices of 500 values made 4096 blocks of two values per thread).  Block (0, 0) also clears the status word.
+__global__ void __launch_bounds__(256) k_logit_keys_static(const float* __restrict__ logits, int vocab,
+                                                           int32_t* __restrict__ status,
                                                            unsigned long long* __restrict__ keys) {
   __shared__ unsigned long long s_best[8];
+  grid_dep_wait();
+  grid_dep_launch();                        // from here on everything before this call in the stream has finished
   const int node = blockIdx.y, chunk = blockIdx.x;
-  const long long v0 = (long long)chunk * vocab / kStaticChunks, v1 = (long long)(chunk + 1) * vocab / kStaticChunks;
+  if (node == 0 && chunk == 0 && threadIdx.x == 0) status[0] = 0;
+  const int v0 = (int)((long long)chunk * vocab / gridDim.x), v1 = (int)((long long)(chunk + 1) * vocab / gridDim.x);
   const float* row = logits + (size_t)node * vocab;
   unsigned long long best = 0ull;
-  for (long long v = v0 + threadIdx.x; v < v1; v += 256) {
+#pragma unroll 8
+  for (int v = v0 + threadIdx.x; v < v1; v += 256) {
     const unsigned long long key = pack_max_key(row[v], (uint32_t)v);
     best = key > best ? key : best;
   }
@@ -47,23 +55,23 @@ __global__ void __launch_bounds__(256) k_logit_keys_static(const float* __restri
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < 8; ++w) best = s_best[w] > best ? s_best[w] : best;
-    keys[(size_t)chunk * SPECASR_MAX_NODES + node] = best;      // 0 = empty slice (vocab < kStaticChunks)
+    keys[(size_t)chunk * SPECASR_MAX_NODES + node] = best;      // 0 = empty slice (fewer tokens than slices)
   }
-  (void)n;
 }
 
+// Accept rule on the slices' candidates.  The tree is read and checked while the candidates are still being computed.
 __global__ void __launch_bounds__(256) k_accept_static(int32_t* __restrict__ status,
-                                                       const unsigned long long* __restrict__ keys,
+                                                       const unsigned long long* __restrict__ keys, int chunks,
                                                        const int32_t* __restrict__ tokens,
                                                        const int32_t* __restrict__ parent, int n, int vocab,
                                                        int32_t* __restrict__ out_argmax,
                                                        int32_t* __restrict__ out_accept_len,
                                                        int32_t* __restrict__ out_path, int32_t* __restrict__ out_bonus) {
-  __shared__ int s_arg[SPECASR_MAX_NODES];
-  __shared__ int s_depth[SPECASR_MAX_NODES];
+  __shared__ int s_arg[SPECASR_MAX_NODES], s_parent[SPECASR_MAX_NODES], s_token[SPECASR_MAX_NODES];
   __shared__ unsigned int s_best;
   __shared__ int s_bad;
   const int i = threadIdx.x;
+  grid_dep_launch();
   if (i == 0) {
     s_bad = 0;
     s_best = 0u;
@@ -71,9 +79,12 @@ __global__ void __launch_bounds__(256) k_accept_static(int32_t* __restrict__ sta
   __syncthreads();
   if (i < n) {
     const int p = parent[i], t = tokens[i];
+    s_parent[i] = p;
+    s_token[i] = t;
     if ((i == 0 ? p != -1 : (p < 0 || p >= i)) || t < 0 || t >= vocab) atomicOr(&s_bad, 1);
   }
   __syncthreads();
+  grid_dep_wait();
   if (s_bad) {
     if (i < n) {
       out_argmax[i] = -1;
@@ -88,28 +99,26 @@ __global__ void __launch_bounds__(256) k_accept_static(int32_t* __restrict__ sta
   }
   if (i < n) {
     unsigned long long best = 0ull;
-    for (int c = 0; c < kStaticChunks; ++c) {
-      const unsigned long long v = keys[(size_t)c * SPECASR_MAX_NODES + i];
+#pragma unroll 8
+    for (int c = 0; c < chunks; ++c) {
+      const unsigned long long v = __ldcg(keys + (size_t)c * SPECASR_MAX_NODES + i);
       best = v > best ? v : best;
     }
     const int tok = (int)(0xFFFFFFFFu - (unsigned int)(best & 0xFFFFFFFFull));
     s_arg[i] = tok;
     out_argmax[i] = tok;
     out_path[i] = -1;
-    int d = 0;
-    for (int j = i; j > 0 && d <= n; j = parent[j]) ++d;     // parent[j] < j was checked: the walk ends
-    s_depth[i] = d;
   }
   __syncthreads();
   if (i < n) {
     bool ok = true;
-    int steps = 0;
-    for (int j = i; j > 0 && steps <= n; ++steps) {
-      const int p = parent[j];
-      ok = ok && (tokens[j] == s_arg[p]);
+    int d = 0;
+    for (int j = i; j > 0 && d <= n; ++d) {                      // parent[j] < j was checked: the walk ends
+      const int p = s_parent[j];
+      ok = ok && (s_token[j] == s_arg[p]);
       j = p;
     }
-    if (ok) atomicMax(&s_best, ((unsigned int)s_depth[i] << 16) | (unsigned int)(0xFFFF - i));
+    if (ok) atomicMax(&s_best, ((unsigned int)d << 16) | (unsigned int)(0xFFFF - i));
   }
   __syncthreads();
   if (i == 0) {
@@ -120,7 +129,7 @@ __global__ void __launch_bounds__(256) k_accept_static(int32_t* __restrict__ sta
     int j = best;
     for (int k = a; k >= 0 && j >= 0; --k) {
       out_path[k] = j;
-      j = parent[j];
+      j = s_parent[j];
     }
   }
 }
@@ -169,16 +178,14 @@ extern "C" specasr_status specasr_accept_logits_static(const float* logits, int3
   cudaStream_t s = (cudaStream_t)stream;
   int32_t* status = (int32_t*)base;
   unsigned long long* keys = (unsigned long long*)((unsigned char*)base + kStaticCtlBytes);
-  // the array keeps whatever the previous call left: the status word must start at zero; the key slots
-  // of nodes 0..n-1 are all rewritten by the first kernel, the others are never read
-  e = cudaMemsetAsync(status, 0, kStaticCtlBytes, s);
-  if (e != cudaSuccess) {
-    set_error("specasr_accept_logits_static: cudaMemsetAsync failed: %s", cudaGetErrorString(e));
-    return SPECASR_ERR_CUDA;
-  }
-  k_logit_keys_static<<<dim3(kStaticChunks, n_nodes), 256, 0, s>>>(logits, vocab, n_nodes, keys);
-  k_accept_static<<<1, 256, 0, s>>>(status, keys, tokens, parent_idx, n_nodes, vocab, out_argmax, out_accept_len,
-                                    out_path, out_bonus);
+  // the array keeps whatever the previous call left: the first kernel clears the status word and rewrites the key slots
+  // that the second one reads
+  int chunks = (4 * 148 + n_nodes - 1) / n_nodes;
+  if (chunks > kStaticChunks) chunks = kStaticChunks;
+  if (chunks > (vocab + 1023) / 1024) chunks = (vocab + 1023) / 1024;        // at least four values per thread
+  launch_pdl(k_logit_keys_static, dim3(chunks, n_nodes), dim3(256), 0, s, logits, vocab, status, keys);
+  launch_pdl(k_accept_static, dim3(1), dim3(256), 0, s, status, keys, chunks, tokens, parent_idx, n_nodes, vocab, out_argmax,
+             out_accept_len, out_path, out_bonus);
   e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_error("specasr_accept_logits_static: launch failed: %s", cudaGetErrorString(e));

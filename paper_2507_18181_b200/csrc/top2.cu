@@ -5,6 +5,8 @@
 //
 // One block per row.  Every thread scans a strided part of the row once, keeping its two largest packed
 // (ordered logit, ~token id) keys and an online (max, sum of exp) pair; warps and then the block merge those.
+#include <cooperative_groups.h>
+
 #include "internal.h"
 #include "device_utils.cuh"
 
@@ -34,53 +36,76 @@ __device__ __forceinline__ void lse_merge(float& m, float& s, float m2, float s2
   m = mm;
 }
 
+// One cluster of CTAs per row: each takes a slice of the vocabulary, the partial results meet in the first CTA's shared
+// memory and are merged in slice order.  Bound by the latency of a slice, not by bandwidth: with one block per row each
+// thread ran through 125 dependent (max, sum) updates of a 32000-token row; a thread now loads eight values at a time,
+// takes their maximum first, and a row is spread over up to eight SMs.
+constexpr int kTop2Cluster = 8;          // CTAs per row, at most
+struct Top2Part {
+  Top2 t;
+  float m, s;
+};
+__device__ __forceinline__ void top2_merge(Top2Part& a, const Top2Part& b) {
+  top2_push(a.t, b.t.a);
+  top2_push(a.t, b.t.b);
+  lse_merge(a.m, a.s, b.m, b.s);
+}
 __global__ void __launch_bounds__(256) k_top2_probs(const float* __restrict__ logits, int vocab,
                                                     int32_t* __restrict__ out_ids, float* __restrict__ out_probs) {
-  __shared__ Top2 s_top[8];
-  __shared__ float s_m[8], s_s[8];
+  namespace cg = cooperative_groups;
+  __shared__ Top2Part s_warp[8];
+  __shared__ Top2Part s_part[kTop2Cluster];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank(), parts = (int)cluster.num_blocks();
+  const int row_id = blockIdx.x / parts;
   grid_dep_launch();
   grid_dep_wait();
-  const float* row = logits + (size_t)blockIdx.x * vocab;
-  Top2 t{0ull, 0ull};
-  float m = -INFINITY, s = 0.f;
-  for (int v = threadIdx.x; v < vocab; v += 256) {
-    const float x = row[v];
-    top2_push(t, pack_max_key(x, (uint32_t)v));
-    if (x > m) {
-      s = s * expf(m - x) + 1.f;       // expf(-inf) = 0 covers the first element
-      m = x;
-    } else {
-      s += expf(x - m);
-    }
+  const float* row = logits + (size_t)row_id * vocab;
+  const int v0 = (int)((long long)rank * vocab / parts), v1 = (int)((long long)(rank + 1) * vocab / parts);
+  Top2Part p{{0ull, 0ull}, -INFINITY, 0.f};
+  for (int base = v0 + threadIdx.x; base < v1; base += 256 * 8) {
+    float x[8];
+    float top = p.m;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = base + u * 256 < v1 ? row[base + u * 256] : -INFINITY;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) top = fmaxf(top, x[u]);
+    p.s *= expf(p.m - top);                 // expf(-inf) = 0 covers the first values
+    p.m = top;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (base + u * 256 < v1) {
+        p.s += expf(x[u] - top);
+        top2_push(p.t, pack_max_key(x[u], (uint32_t)(base + u * 256)));
+      }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long oa = __shfl_xor_sync(0xFFFFFFFFu, t.a, o), ob = __shfl_xor_sync(0xFFFFFFFFu, t.b, o);
-    top2_push(t, oa);
-    top2_push(t, ob);
-    const float om = __shfl_xor_sync(0xFFFFFFFFu, m, o), os = __shfl_xor_sync(0xFFFFFFFFu, s, o);
-    lse_merge(m, s, om, os);
+    Top2Part q;
+    q.t.a = __shfl_xor_sync(0xFFFFFFFFu, p.t.a, o);
+    q.t.b = __shfl_xor_sync(0xFFFFFFFFu, p.t.b, o);
+    q.m = __shfl_xor_sync(0xFFFFFFFFu, p.m, o);
+    q.s = __shfl_xor_sync(0xFFFFFFFFu, p.s, o);
+    top2_merge(p, q);
   }
-  const int warp = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) {
-    s_top[warp] = t;
-    s_m[warp] = m;
-    s_s[warp] = s;
-  }
+  if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = p;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) {
-      top2_push(t, s_top[w].a);
-      top2_push(t, s_top[w].b);
-      lse_merge(m, s, s_m[w], s_s[w]);
-    }
+    for (int w = 1; w < 8; ++w) top2_merge(p, s_warp[w]);
+    *cluster.map_shared_rank(&s_part[rank], 0) = p;
+  }
+  cluster.sync();                            // afterwards only the first CTA reads, and only its own shared memory
+  if (rank == 0 && threadIdx.x == 0) {
+    p = s_part[0];
+    for (int q = 1; q < parts; ++q) top2_merge(p, s_part[q]);
+    Top2& t = p.t;
     if (t.b == 0ull) t.b = t.a;                    // a one-token vocabulary
-    int32_t* ids = out_ids + (size_t)blockIdx.x * 2;
-    float* pr = out_probs + (size_t)blockIdx.x * 2;
+    int32_t* ids = out_ids + (size_t)row_id * 2;
+    float* pr = out_probs + (size_t)row_id * 2;
     ids[0] = (int32_t)(0xFFFFFFFFu - (uint32_t)(t.a & 0xFFFFFFFFull));
     ids[1] = (int32_t)(0xFFFFFFFFu - (uint32_t)(t.b & 0xFFFFFFFFull));
-    pr[0] = expf(key_value(t.a) - m) / s;
-    pr[1] = expf(key_value(t.b) - m) / s;
+    pr[0] = expf(key_value(t.a) - p.m) / p.s;
+    pr[1] = expf(key_value(t.b) - p.m) / p.s;
   }
 }
 
@@ -164,7 +189,10 @@ extern "C" specasr_status specasr_top2_probs(const float* logits, int32_t n_rows
     set_error("specasr_top2_probs: n_rows = %d and vocab = %d must be positive", n_rows, vocab);
     return SPECASR_ERR_INVALID_ARG;
   }
-  launch_pdl(k_top2_probs, dim3(n_rows), dim3(256), 0, (cudaStream_t)stream, logits, vocab, out_ids, out_probs);
+  int parts = 1;                               // CTAs per row: at least eight values per thread
+  while (parts < kTop2Cluster && vocab / (2 * parts) >= 2048) parts *= 2;
+  launch_pdl_cluster(k_top2_probs, dim3(parts * n_rows), dim3(256), parts, 0, (cudaStream_t)stream, logits, vocab, out_ids,
+                     out_probs);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_error("specasr_top2_probs: %s", cudaGetErrorString(e));
