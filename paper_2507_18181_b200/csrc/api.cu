@@ -304,7 +304,7 @@ extern "C" specasr_status specasr_kv_create(const specasr_model* m, void* k_pool
   kv->len_host = 0;
   kv->len_exact = true;
   kv->len_upper = 0;
-  kv->pinned = nullptr;
+  kv->pinned = kv->pinned_dev = nullptr;
   kv->len_event_pending = false;
   kv->launches = 0;
   kv->gemm_epoch = 0;
@@ -314,6 +314,7 @@ extern "C" specasr_status specasr_kv_create(const specasr_model* m, void* k_pool
   kv->trace.buf = nullptr;
   kv->trace.cap = 0;
   cudaError_t e = cudaHostAlloc(&kv->pinned, 4 * sizeof(int32_t), cudaHostAllocDefault);
+  if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&kv->pinned_dev, kv->pinned, 0);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&kv->len_event, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMemset(kv->ws.ctl, 0, sizeof(int32_t) * kCtlWords);
   if (e == cudaSuccess) e = cudaMemset(kv->ws.fixFlag, 0, sizeof(int32_t) * m->n_sm);
@@ -407,8 +408,7 @@ extern "C" specasr_status specasr_profile_read(specasr_kv* kv, double* out_ms, i
   return SPECASR_OK;
 }
 
-// The host learns the committed length lazily: a commit enqueues a copy of the device length word
-// into pinned memory followed by an event.
+// The host learns the committed length lazily: a commit's kernel writes it into pinned memory, and an event follows.
 static void refresh_len(specasr_kv* kv, bool wait) {
   if (!kv->len_event_pending) return;
   cudaError_t q = wait ? cudaEventSynchronize(kv->len_event) : cudaEventQuery(kv->len_event);
@@ -614,7 +614,6 @@ static specasr_status prefill_common(specasr_model* m, specasr_kv* kv, const flo
   }
   // The device may have refused a chunk (a token id outside the vocabulary): the host learns the length the same
   // lazy way as after a commit, so that specasr_kv_length reports what the device holds.
-  CUDA_TRY(cudaMemcpyAsync(kv->pinned, kv->ws.ctl + CTL_LEN, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaEventRecord(kv->len_event, s));
   kv->len_event_pending = true;           // len_host stays the optimistic value (an upper bound) until the copy lands
   CUDA_TRY(cudaGetLastError());
@@ -663,8 +662,7 @@ static specasr_status verify_tree_impl(specasr_model* m, specasr_kv* kv, const i
               "64 nodes)");
     return SPECASR_ERR_UNSUPPORTED;
   }
-  launch_tree_prep(kv, tab, tokens, parent_idx, s);
-  launch_embed_tokens(kv, tab, n_nodes, tokens, s);
+  launch_tree_prep(kv, tab, n_nodes, tokens, parent_idx, nullptr, s);
   run_stack(m, kv, tab, n_nodes, att_tc, kv->ws.ctl, true, out_logits, want_top2, s);
   launch_accept(kv, tab, nullptr, tokens, parent_idx, lm_tiles_of(m), out_argmax, out_accept_len, out_path, out_bonus, s);
   if (want_top2) launch_top2_from_tiles(kv, tab, nullptr, n_nodes, lm_tiles_of(m), out_top2_ids, out_top2_probs, s);
@@ -764,14 +762,12 @@ static specasr_status verify_batch_impl(specasr_model* m, int32_t batch, specasr
   attention_tc_plan(m, &tab, len_upper);
   cudaStream_t s = (cudaStream_t)stream;
   int32_t* ctl_shared = wk->ws.ctl + kCtlBatch;
-  CUDA_TRY(cudaMemsetAsync(ctl_shared, 0, sizeof(int32_t) * 4, s));
   const bool want_top2 = out_top2_ids != nullptr;
   if (want_top2 && !fused_stack_supported(wk, total, true)) {
     set_error("%s: the top-2 epilogue needs the fused layer stack (at most 64 nodes in all)", who);
     return SPECASR_ERR_UNSUPPORTED;
   }
-  launch_tree_prep(wk, tab, tokens, parent_idx, s);
-  launch_embed_tokens(wk, tab, total, tokens, s);
+  launch_tree_prep(wk, tab, total, tokens, parent_idx, ctl_shared, s);
   run_stack(m, wk, tab, total, true, ctl_shared, true, out_logits, want_top2, s);
   launch_accept(wk, tab, ctl_shared, tokens, parent_idx, lm_tiles_of(m), out_argmax, out_accept_len, out_path, out_bonus,
                 s);
@@ -820,7 +816,6 @@ extern "C" specasr_status specasr_commit_kv(specasr_model* m, specasr_kv* kv, co
   cudaStream_t s = (cudaStream_t)stream;
   refresh_len(kv, false);
   launch_commit(kv, path, accept_len, s);
-  CUDA_TRY(cudaMemcpyAsync(kv->pinned, kv->ws.ctl + CTL_LEN, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaEventRecord(kv->len_event, s));
   kv->len_event_pending = true;
   kv->len_exact = false;

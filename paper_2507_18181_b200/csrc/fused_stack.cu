@@ -92,7 +92,7 @@ struct StackParams {
   int n, n_pad, n_alloc, stages, stage_bytes, ring_bytes;
   int splits_qkv, splits_o, splits_down, epoch0, want_head, group, nodes_per_tile, whole_gu, whole_lm;
   int32_t* ctl;                         // control block whose status word ends the call
-  int32_t* sync;                        // [steps of the call] arrival counters, zeroed before the launch
+  int32_t* sync;                        // [steps of the call] arrival counters, cleared by the kernel that prepares the rows
   float* X;
   float* P;
   float* fixP;
@@ -320,6 +320,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_launch_dependents();                              // the accept kernel's launch overlaps; it waits for this grid's end
   const uint32_t tmem_base = sc->tmem_base;
   volatile int* abort = &sc->abort;
   int32_t* status = p.ctl + CTL_STATUS;
@@ -1231,11 +1232,9 @@ bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, i
 #pragma unroll 1
   for (int b = 16; b < n_pad; b <<= 1) ++idx;
   LaunchScope scope(wk, SPECASR_KIND_STACK, s);
-  cudaError_t e = cudaMemsetAsync(wk->ws.sync, 0, fused_stack_sync_bytes(m), s);
-  if (e == cudaSuccess) {
-    if (c.head_dim == 64) e = launch_dh<64>(wk->tm_H[idx], wk->tm_AO[idx], wk->tm_A[idx], wk->tm_Q, tab, p, m->n_sm, smem, s);
-    else e = launch_dh<128>(wk->tm_H[idx], wk->tm_AO[idx], wk->tm_A[idx], wk->tm_Q, tab, p, m->n_sm, smem, s);
-  }
+  cudaError_t e;                                         // the counters were cleared by the kernel that prepared the rows
+  if (c.head_dim == 64) e = launch_dh<64>(wk->tm_H[idx], wk->tm_AO[idx], wk->tm_A[idx], wk->tm_Q, tab, p, m->n_sm, smem, s);
+  else e = launch_dh<128>(wk->tm_H[idx], wk->tm_AO[idx], wk->tm_A[idx], wk->tm_Q, tab, p, m->n_sm, smem, s);
   if (e != cudaSuccess) {
     set_error("fused layer stack launch failed: %s", cudaGetErrorString(e));
     return false;

@@ -20,7 +20,7 @@ constexpr int kActBoxRows[kActBoxes] = {16, 32, 64, 80, 96, 112, 128};   // toke
 constexpr int kCtlWords = 64;      // int32 control block at the start of the workspace
 
 // control block word indices
-enum { CTL_LEN = 0, CTL_STATUS = 1, CTL_N = 2 };
+enum { CTL_LEN = 0, CTL_STATUS = 1, CTL_N = 2, CTL_DONE = 3 };      // CTL_DONE: blocks of a commit that have finished
 // A second control block (same word layout) at this offset serves the kernels that a batched call runs once
 // over all utterances: its status word only ever records a bounded wait that ran out.
 constexpr int kCtlBatch = 16;
@@ -105,7 +105,8 @@ struct specasr_kv {
   int len_host;             // last length the host knows exactly
   bool len_exact;           // false while a commit's length has not been read back
   int len_upper;            // upper bound of the length
-  int32_t* pinned;          // [4] pinned host words: [0] length, [2] status (1 and 3 unused)
+  int32_t* pinned;          // [4] pinned host words: [0] length, written by the device, [2] status (1 and 3 unused)
+  int32_t* pinned_dev;      // the same memory as the device addresses it
   cudaEvent_t len_event;
   bool len_event_pending;
   int64_t launches;
@@ -223,7 +224,8 @@ Workspace carve_workspace(const specasr_model* m, int n_alloc, void* base);
 int lm_tiles_of(const specasr_model* m);
 
 // ---- kernels_small.cu
-void launch_tree_prep(specasr_kv* wk, const SegTable& t, const int32_t* tokens, const int32_t* parent, cudaStream_t s);
+void launch_tree_prep(specasr_kv* wk, const SegTable& t, int n_total, const int32_t* tokens, const int32_t* parent,
+                      int32_t* ctl_shared, cudaStream_t s);          // + embedding of every row
 void launch_chain_prep(specasr_kv* kv, int n, bool first, cudaStream_t s);
 void launch_embed_tokens(specasr_kv* wk, const SegTable& t, int n_total, const int32_t* tokens, cudaStream_t s);
 void launch_copy_embeds(specasr_kv* kv, const float* embeds, int n, cudaStream_t s);

@@ -9,18 +9,47 @@
 // Tree preparation: validates the parent array, derives depth, position and the ancestor-or-self
 // bitmask of every node (the rows of the 2-D tree attention mask), and sets the status word that
 // every later kernel of the call checks.
-// One block per utterance of the call; tokens / parent / depth / pos / anc are indexed by workspace row.
+// One block per utterance of the call, then one per row, which looks its token up (layer-0 inputs): a bad token is skipped
+// there and refused by its utterance's block.  The first block also clears what the rest of the call counts in: the
+// arrival counters of the fused stack and the status words of a batched call.  (As four launches -- two clears, this, the
+// embedding -- the same took 8 us more of a round.)  tokens / parent / depth / pos / anc are indexed by workspace row.
+__device__ __forceinline__ void embed_row(const bf16* __restrict__ row, int d, float* __restrict__ x) {
+  for (int k = threadIdx.x * 8; k < d; k += blockDim.x * 8) {
+    const uint4 v = *reinterpret_cast<const uint4*>(row + k);
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    float4 a, b;
+    a.x = bf16lo_to_f32(w[0]); a.y = bf16hi_to_f32(w[0]);
+    a.z = bf16lo_to_f32(w[1]); a.w = bf16hi_to_f32(w[1]);
+    b.x = bf16lo_to_f32(w[2]); b.y = bf16hi_to_f32(w[2]);
+    b.z = bf16lo_to_f32(w[3]); b.w = bf16hi_to_f32(w[3]);
+    *reinterpret_cast<float4*>(x + k) = a;
+    *reinterpret_cast<float4*>(x + k + 4) = b;
+  }
+}
+__device__ __forceinline__ void clear_counters(int32_t* __restrict__ sync, int words) {
+  for (int k = threadIdx.x; k < words; k += blockDim.x) sync[k] = 0;
+}
 __global__ void k_tree_prep(const __grid_constant__ SegTable tab, const int32_t* __restrict__ tokens,
                             const int32_t* __restrict__ parent, int vocab, int32_t* __restrict__ depth,
-                            int32_t* __restrict__ pos, unsigned long long* __restrict__ anc SPECASR_TRACE_PARAM) {
+                            int32_t* __restrict__ pos, unsigned long long* __restrict__ anc, const bf16* __restrict__ E, int d,
+                            float* __restrict__ X, int32_t* __restrict__ sync, int sync_words,
+                            int32_t* __restrict__ ctl_shared SPECASR_TRACE_PARAM) {
   __shared__ int s_bad;
   __shared__ int s_parent[SPECASR_MAX_NODES];     // the ancestor walk would otherwise be a chain of global loads
   SPECASR_TRACE_SCOPE(tr, SPECASR_KIND_PREP);
   const int i = threadIdx.x;
+  if (blockIdx.x >= tab.count) {
+    grid_dep_launch();
+    grid_dep_wait();
+    SPECASR_TRACE_MARK();
+    const int row = blockIdx.x - tab.count, tok = tokens[row];
+    if (tok >= 0 && tok < vocab) embed_row(E + (size_t)tok * d, d, X + (size_t)row * d);
+    return;
+  }
   const SegDev& sg = tab.seg[blockIdx.x];
   int32_t* ctl = sg.ctl;
   const int n = sg.n, capacity = sg.capacity;
-  if (tokens) tokens += sg.row0;
+  tokens += sg.row0;
   parent += sg.row0;
   depth += sg.row0;
   pos += sg.row0;
@@ -28,13 +57,17 @@ __global__ void k_tree_prep(const __grid_constant__ SegTable tab, const int32_t*
   grid_dep_launch();
   grid_dep_wait();
   SPECASR_TRACE_MARK();
+  if (blockIdx.x == 0) {
+    clear_counters(sync, sync_words);
+    if (ctl_shared && i < 4) ctl_shared[i] = 0;
+  }
   if (i == 0) s_bad = 0;
   __syncthreads();
   const int L = ctl[CTL_LEN];
   if (i < n) {
     const int p = parent[i];
     s_parent[i] = p;
-    const int t = tokens ? tokens[i] : 0;
+    const int t = tokens[i];
     const bool bad = (i == 0 ? p != -1 : (p < 0 || p >= i)) || t < 0 || t >= vocab;
     if (bad) atomicOr(&s_bad, 1);
   }
@@ -69,10 +102,12 @@ __global__ void k_tree_prep(const __grid_constant__ SegTable tab, const int32_t*
 // Only the first chunk of a context-fill call starts from a clean status: a chunk that was refused (capacity, a
 // token id outside the vocabulary) keeps every later chunk of the same call from running on top of the gap.
 __global__ void k_chain_prep(int32_t* __restrict__ ctl, int n, int capacity, int first, int32_t* __restrict__ depth,
-                             int32_t* __restrict__ pos, unsigned long long* __restrict__ anc) {
+                             int32_t* __restrict__ pos, unsigned long long* __restrict__ anc, int32_t* __restrict__ sync,
+                             int sync_words) {
   const int i = threadIdx.x;
   grid_dep_launch();
   grid_dep_wait();
+  clear_counters(sync, sync_words);
   if (!first && ctl[CTL_STATUS] != 0) return;
   const int L = ctl[CTL_LEN];
   if (L < 0 || L + n > capacity) {
@@ -97,10 +132,12 @@ __global__ void k_chain_prep(int32_t* __restrict__ ctl, int n, int capacity, int
   }
 }
 
-void launch_tree_prep(specasr_kv* wk, const SegTable& t, const int32_t* tokens, const int32_t* parent, cudaStream_t s) {
+void launch_tree_prep(specasr_kv* wk, const SegTable& t, int n_total, const int32_t* tokens, const int32_t* parent,
+                      int32_t* ctl_shared, cudaStream_t s) {
   LaunchScope scope(wk, SPECASR_KIND_PREP, s);
-  launch_pdl(k_tree_prep, dim3(t.count), dim3(256), 0, s, t, tokens, parent, wk->m->cfg.vocab, wk->ws.depth,
-             wk->ws.pos, wk->ws.anc SPECASR_TRACE_ARG(wk));
+  launch_pdl(k_tree_prep, dim3(t.count + n_total), dim3(256), 0, s, t, tokens, parent, wk->m->cfg.vocab, wk->ws.depth,
+             wk->ws.pos, wk->ws.anc, wk->m->embed, wk->m->cfg.d_model, wk->ws.X, wk->ws.sync,
+             (int)(fused_stack_sync_bytes(wk->m) / sizeof(int32_t)), ctl_shared SPECASR_TRACE_ARG(wk));
 }
 
 void launch_chain_prep(specasr_kv* kv, int n, bool first, cudaStream_t s) {
@@ -108,7 +145,8 @@ void launch_chain_prep(specasr_kv* kv, int n, bool first, cudaStream_t s) {
   int cap = kv->max_pages * m->cfg.page_size;
   if (m->cfg.max_positions < cap) cap = m->cfg.max_positions;
   LaunchScope scope(kv, SPECASR_KIND_PREP, s);
-  launch_pdl(k_chain_prep, dim3(1), dim3(256), 0, s, kv->ws.ctl, n, cap, first ? 1 : 0, kv->ws.depth, kv->ws.pos, kv->ws.anc);
+  launch_pdl(k_chain_prep, dim3(1), dim3(256), 0, s, kv->ws.ctl, n, cap, first ? 1 : 0, kv->ws.depth, kv->ws.pos, kv->ws.anc,
+             kv->ws.sync, (int)(fused_stack_sync_bytes(m) / sizeof(int32_t)));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -137,19 +175,7 @@ __global__ void k_embed_tokens(const __grid_constant__ SegTable tab, const int32
     if (threadIdx.x == 0) ctl[CTL_STATUS] = SPECASR_ERR_INVALID_TREE;
     return;
   }
-  const bf16* row = E + (size_t)tok * d;
-  float* x = X + (size_t)i * d;
-  for (int k = threadIdx.x * 8; k < d; k += blockDim.x * 8) {
-    const uint4 v = *reinterpret_cast<const uint4*>(row + k);
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    float4 a, b;
-    a.x = bf16lo_to_f32(w[0]); a.y = bf16hi_to_f32(w[0]);
-    a.z = bf16lo_to_f32(w[1]); a.w = bf16hi_to_f32(w[1]);
-    b.x = bf16lo_to_f32(w[2]); b.y = bf16hi_to_f32(w[2]);
-    b.z = bf16lo_to_f32(w[3]); b.w = bf16hi_to_f32(w[3]);
-    *reinterpret_cast<float4*>(x + k) = a;
-    *reinterpret_cast<float4*>(x + k + 4) = b;
-  }
+  embed_row(E + (size_t)tok * d, d, X + (size_t)i * d);
 }
 
 __global__ void k_copy_embeds(const int32_t* __restrict__ ctl, const float* __restrict__ src, int d,
@@ -606,11 +632,12 @@ void launch_accept(specasr_kv* wk, const SegTable& t, const int32_t* ctl_shared,
 
 // ------------------------------------------------------------------------------------------------
 // Cache length bookkeeping.
-__global__ void k_advance_len(int32_t* ctl, int n) {
+// `host_len` is the pinned host word from which the host learns the length once the event behind the kernel has passed.
+__global__ void k_advance_len(int32_t* ctl, int n, int32_t* host_len) {
   grid_dep_launch();
   grid_dep_wait();
-  if (ctl[CTL_STATUS] != 0) return;
-  ctl[CTL_LEN] += n;
+  if (ctl[CTL_STATUS] == 0) ctl[CTL_LEN] += n;
+  *host_len = ctl[CTL_LEN];
 }
 __global__ void k_set_len(int32_t* ctl, int len) {
   grid_dep_launch();
@@ -621,7 +648,7 @@ __global__ void k_set_len(int32_t* ctl, int len) {
 }
 void launch_advance_len(specasr_kv* kv, int n, cudaStream_t s) {
   LaunchScope scope(kv, SPECASR_KIND_COMMIT, s);
-  launch_pdl(k_advance_len, dim3(1), dim3(1), 0, s, kv->ws.ctl, n);
+  launch_pdl(k_advance_len, dim3(1), dim3(1), 0, s, kv->ws.ctl, n, kv->pinned_dev);
 }
 void launch_set_len(specasr_kv* kv, int len, cudaStream_t s) {
   LaunchScope scope(kv, SPECASR_KIND_COMMIT, s);
@@ -632,59 +659,63 @@ void launch_set_len(specasr_kv* kv, int len, cudaStream_t s) {
 // Commit: slot L+j <- slot L+path[j], j ascending.  path[j] >= j and strictly increasing, so a
 // destination is never the source of a later move; each thread owns one 16-byte column of one
 // (layer, pool, kv head, plane) and walks j in order, which makes the in-place copy safe.
-__global__ void __launch_bounds__(256) k_commit(const int32_t* __restrict__ ctl, const int32_t* __restrict__ path,
+// The last block to finish moves the length on and hands it to the host (a launch and a copy of their own before: 4 us
+// per utterance and round).
+__global__ void __launch_bounds__(256) k_commit(int32_t* __restrict__ ctl, const int32_t* __restrict__ path,
                                                 const int32_t* __restrict__ accept_len, bf16* __restrict__ k_pool,
                                                 bf16* __restrict__ v_pool, const int32_t* __restrict__ page_table,
-                                                int n_pages, int Hkv, int page_size, int dh) {
+                                                int n_pages, int Hkv, int page_size, int dh, int32_t* host_len) {
   grid_dep_launch();
   grid_dep_wait();
   __shared__ int s_path[SPECASR_MAX_NODES];      // read once, side by side, instead of one dependent load per step
   const int a = accept_len[0];
   const int n = ctl[CTL_N];
-  if (ctl[CTL_STATUS] != 0 || a < 0 || a >= n) return;
-  for (int j = threadIdx.x; j <= a; j += blockDim.x) s_path[j] = path[j];
-  __syncthreads();
   const int L = ctl[CTL_LEN];
-  const int layer = blockIdx.x;
-  bf16* pool = blockIdx.y == 0 ? k_pool : v_pool;
-  const int chunks_per_row = dh / 8;
-  const int cols = Hkv * 2 * chunks_per_row;
-  for (int c = threadIdx.x; c < cols; c += blockDim.x) {
-    const int kvh = c / (2 * chunks_per_row);
-    const int plane = (c / chunks_per_row) & 1;
-    const int ch = c % chunks_per_row;
-    int prev = 0;
-    for (int j = 1; j <= a; ++j) {
-      const int pj = s_path[j];
-      if (pj <= prev || pj >= n) break;   // not a root path of the pending tree: stop copying
-      prev = pj;
-      if (pj == j) continue;
-      const int src = L + pj, dst = L + j;
-      const bf16* sp = pool + kv_plane_offset(layer, n_pages, Hkv, page_size, dh, page_table[src / page_size], kvh, plane) +
-                       (size_t)(src % page_size) * dh + ch * 8;
-      bf16* dp = pool + kv_plane_offset(layer, n_pages, Hkv, page_size, dh, page_table[dst / page_size], kvh, plane) +
-                 (size_t)(dst % page_size) * dh + ch * 8;
-      *reinterpret_cast<uint4*>(dp) = *reinterpret_cast<const uint4*>(sp);
+  const bool valid = ctl[CTL_STATUS] == 0 && a >= 0 && a < n;      // the same for every block: only the last one writes
+  if (valid) {
+    for (int j = threadIdx.x; j <= a; j += blockDim.x) s_path[j] = path[j];
+    __syncthreads();
+    const int layer = blockIdx.x;
+    bf16* pool = blockIdx.y == 0 ? k_pool : v_pool;
+    const int chunks_per_row = dh / 8;
+    const int cols = Hkv * 2 * chunks_per_row;
+    for (int c = threadIdx.x; c < cols; c += blockDim.x) {
+      const int kvh = c / (2 * chunks_per_row);
+      const int plane = (c / chunks_per_row) & 1;
+      const int ch = c % chunks_per_row;
+      int prev = 0;
+      for (int j = 1; j <= a; ++j) {
+        const int pj = s_path[j];
+        if (pj <= prev || pj >= n) break;   // not a root path of the pending tree: stop copying
+        prev = pj;
+        if (pj == j) continue;
+        const int src = L + pj, dst = L + j;
+        const bf16* sp = pool + kv_plane_offset(layer, n_pages, Hkv, page_size, dh, page_table[src / page_size], kvh, plane) +
+                         (size_t)(src % page_size) * dh + ch * 8;
+        bf16* dp = pool + kv_plane_offset(layer, n_pages, Hkv, page_size, dh, page_table[dst / page_size], kvh, plane) +
+                   (size_t)(dst % page_size) * dh + ch * 8;
+        *reinterpret_cast<uint4*>(dp) = *reinterpret_cast<const uint4*>(sp);
+      }
+    }
+  }
+  __syncthreads();                          // every thread has read the control words
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const int total = (int)(gridDim.x * gridDim.y);
+    if (atomicAdd(ctl + CTL_DONE, 1) == total - 1) {
+      ctl[CTL_DONE] = 0;
+      if (valid) {
+        ctl[CTL_LEN] = L + a + 1;
+        ctl[CTL_N] = 0;
+      }
+      *host_len = valid ? L + a + 1 : L;
     }
   }
 }
 
-__global__ void k_commit_finish(int32_t* ctl, const int32_t* __restrict__ accept_len) {
-  grid_dep_launch();
-  grid_dep_wait();
-  const int a = accept_len[0];
-  const int n = ctl[CTL_N];
-  if (ctl[CTL_STATUS] != 0 || a < 0 || a >= n) return;
-  ctl[CTL_LEN] += a + 1;
-  ctl[CTL_N] = 0;
-}
-
 void launch_commit(specasr_kv* kv, const int32_t* path, const int32_t* accept_len, cudaStream_t s) {
   const specasr_model_config& c = kv->m->cfg;
-  dim3 grid(c.n_layers, 2);
   LaunchScope scope(kv, SPECASR_KIND_COMMIT, s);
-  launch_pdl(k_commit, grid, dim3(256), 0, s, kv->ws.ctl, path, accept_len, kv->k_pool, kv->v_pool, kv->page_table, kv->n_pages,
-                                c.n_kv_heads, c.page_size, c.head_dim);
-  launch_pdl(k_commit_finish, dim3(1), dim3(1), 0, s, kv->ws.ctl, accept_len);
-  kv->launches++;
+  launch_pdl(k_commit, dim3(c.n_layers, 2), dim3(256), 0, s, kv->ws.ctl, path, accept_len, kv->k_pool, kv->v_pool,
+             kv->page_table, kv->n_pages, c.n_kv_heads, c.page_size, c.head_dim, kv->pinned_dev);
 }
