@@ -328,7 +328,7 @@ extern "C" specasr_status specasr_kv_create(const specasr_model* m, void* k_pool
   if (m->cfg.gemm_path == 0) {
     const specasr_model_config& c = m->cfg;
     bool ok = true;
-    for (int i = 0, b = 16; i < 3 && b <= kv->n_alloc && ok; ++i, b <<= 1) {
+    for (int i = 0, b = 16; i < 4 && b <= kv->n_alloc && ok; ++i, b += 16) {
       ok = make_act_map(&kv->tm_H[i], kv->ws.H, c.d_model, kv->n_alloc, b, 2) &&
            make_act_map(&kv->tm_AO[i], kv->ws.AO, m->q_dim, kv->n_alloc, b, 2) &&
            make_act_map(&kv->tm_A[i], kv->ws.A, c.ffn, kv->n_alloc, b, 2);

@@ -117,9 +117,9 @@ struct specasr_kv {
   std::vector<int> prof_kinds;
   size_t prof_used;                       // launches recorded since the last read
   TraceBuf trace;                         // device-side trace, off unless specasr_trace_set was called
-  // activation TMA descriptors (tcgen05 path): boxes of both planes for the fused stack, one per height 16 << i, and
+  // activation TMA descriptors (tcgen05 path): boxes of both planes for the fused stack, one per height 16 (i + 1), and
   // boxes of one plane for the separate projections, one per height in kActBoxRows
-  CUtensorMap tm_H[3], tm_AO[3], tm_A[3];
+  CUtensorMap tm_H[4], tm_AO[4], tm_A[4];
   CUtensorMap tm_H1[kActBoxes], tm_AO1[kActBoxes], tm_A1[kActBoxes];
   // tensor-core attention: rotated queries and the two pools
   bool attn_tc;

@@ -33,6 +33,7 @@ class _SharpStore(gen.WeightStore):
 @pytest.mark.parametrize("cfg_name,context,nodes,page_size,sharp", [
     ("small", 15, 1, 16, 1), ("small", 47, 17, 16, 1), ("small", 63, 2, 16, 1), ("small", 112, 16, 16, 1),
     ("tiny", 49, 15, 16, 1), ("tiny", 191, 64, 16, 1), ("tiny", 130, 63, 48, 1), ("small", 320, 70, 80, 1),
+    ("small", 100, 33, 16, 1), ("tiny", 100, 48, 16, 1), ("small", 100, 49, 16, 1),      # row padding 32 | 48 | 64
     ("tiny", 400, 40, 16, 8), ("small", 400, 40, 16, 8), ("small", 700, 130, 16, 8), ("tiny", 701, 256, 16, 8),
 ])
 def test_ranges_and_rescaling_match_the_oracle(cfg_name, context, nodes, page_size, sharp):
