@@ -30,6 +30,18 @@ __device__ __forceinline__ void split2_pack(float a, float b, uint32_t& hi, uint
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
+// SiLU(gate) * up of 16 tokens of one feature whose gate row is held by the even lane of a pair and whose up row by the odd
+// one (v = this lane's row).  The even lane finishes tokens 0..7, the odd lane tokens 8..15: each sends the half that it
+// does not need, so that nothing is computed twice.
+__device__ __forceinline__ void swiglu_pair(const float* v, bool odd, float* a) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const float other = __shfl_xor_sync(0xFFFFFFFFu, odd ? v[j] : v[8 + j], 1);
+    const float gate = odd ? other : v[j], up = odd ? v[8 + j] : other;
+    a[j] = __fdividef(gate, 1.f + __expf(-gate)) * up;
+  }
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);

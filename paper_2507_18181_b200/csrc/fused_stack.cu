@@ -788,22 +788,17 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
 #pragma unroll
             for (int j = 0; j < 16; ++j) v[j] *= sc->inv[c0 + j];
             if (swiglu) {
-              // rows 2f / 2f + 1 of the tile are gate / up of feature f: the even lane keeps the hi plane of the
-              // product, the odd lane the lo plane, staged in shared memory for 16-byte global stores
-              float a[16];
+              // rows 2f / 2f + 1 of the tile are gate / up of feature f: the even lane of the pair finishes eight of the
+              // tokens, the odd lane the other eight; both planes are staged in shared memory for 16-byte global stores
+              float a[8];
+              swiglu_pair(v, (lane & 1) != 0, a);
+              bf16* st = epi_stage + (size_t)(c0 + (lane & 1) * 8) * 64 + (row >> 1);
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const float other = __shfl_xor_sync(0xFFFFFFFFu, v[j], 1);
-                const float gt = (lane & 1) ? other : v[j];
-                const float up = (lane & 1) ? v[j] : other;
-                a[j] = __fdividef(gt, 1.f + __expf(-gt)) * up;
-              }
-              bf16* st = epi_stage + (size_t)(lane & 1) * n_pad * 64 + (size_t)c0 * 64 + (row >> 1);
-#pragma unroll
-              for (int j = 0; j < 16; ++j) {
+              for (int j = 0; j < 8; ++j) {
                 bf16 hi, lo;
                 split_bf16(a[j], hi, lo);
-                st[j * 64] = (lane & 1) ? lo : hi;
+                st[j * 64] = hi;
+                st[n_pad * 64 + j * 64] = lo;
               }
             } else {
 #pragma unroll

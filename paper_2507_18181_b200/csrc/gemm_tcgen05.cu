@@ -285,8 +285,8 @@ __global__ void __launch_bounds__(64 + EPI_THREADS, 1) k_proj(const __grid_const
       int last = pair;
       if (EPI != EPI_PARTIAL && kb0 == 0 && kb1 != KB)
         while (last + 1 < G && (long long)(last + 1) * U / G < (long long)(ptile + 1) * KB) ++last;
-      float pk[16];
-      auto load_parked = [&](int c0) {
+      float pk[16], pk_next[16];                          // parked sums of the next two blocks of this warp
+      auto load_parked = [&](int c0, float* pk) {
 #pragma unroll
         for (int j = 0; j < 16; ++j) pk[j] = 0.f;
         if (c0 < p.n_pad)
@@ -313,7 +313,10 @@ __global__ void __launch_bounds__(64 + EPI_THREADS, 1) k_proj(const __grid_const
         }
         epi_bar();
         if (*abort) ok = false;
-        if (ok) load_parked(c_first);
+        if (ok) {
+          load_parked(c_first, pk);
+          load_parked(c_first + 32, pk_next);
+        }
       }
       if (ok) ok = mbar_wait_relaxed(&sc->acc_full[b], (uint32_t)((seg >> 1) & 1), abort, status);
       ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;     // TMEM loads are warp-wide
@@ -367,26 +370,24 @@ __global__ void __launch_bounds__(64 + EPI_THREADS, 1) k_proj(const __grid_const
             load16(lane_addr, c0, v);
             if (last > pair) {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) v[j] += pk[j];
-              load_parked(c0 + 32);                       // the next block's parked sums travel meanwhile
+              for (int j = 0; j < 16; ++j) {
+                v[j] += pk[j];
+                pk[j] = pk_next[j];
+              }
+              load_parked(c0 + 64, pk_next);              // travels while this block and the next are worked on
             }
             if (EPI == EPI_SWIGLU) {
-              // rows 2f / 2f + 1 of the tile are gate / up of feature f: the even lane keeps the hi plane of
-              // the product, the odd lane the lo plane, staged in shared memory for 16-byte global stores
-              float a[16];
+              // rows 2f / 2f + 1 of the tile are gate / up of feature f: the even lane of the pair finishes eight of the
+              // tokens, the odd lane the other eight; both planes are staged in shared memory for 16-byte global stores
+              float a[8];
+              swiglu_pair(v, (lane & 1) != 0, a);
+              bf16* st = epi_stage + (size_t)(c0 - tc0 + (lane & 1) * 8) * 64 + (row >> 1);
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const float other = __shfl_xor_sync(0xFFFFFFFFu, v[j], 1);
-                const float g = (lane & 1) ? other : v[j];
-                const float up = (lane & 1) ? v[j] : other;
-                a[j] = __fdividef(g, 1.f + __expf(-g)) * up;
-              }
-              bf16* st = epi_stage + (size_t)(lane & 1) * EPI_TOKENS * 64 + (size_t)(c0 - tc0) * 64 + (row >> 1);
-#pragma unroll
-              for (int j = 0; j < 16; ++j) {
+              for (int j = 0; j < 8; ++j) {
                 bf16 hi, lo;
                 split_bf16(a[j], hi, lo);
-                st[j * 64] = (lane & 1) ? lo : hi;
+                st[j * 64] = hi;
+                st[EPI_TOKENS * 64 + j * 64] = lo;
               }
             } else if (EPI == EPI_ARGMAX) {
 #pragma unroll
