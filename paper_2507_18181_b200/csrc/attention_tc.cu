@@ -37,7 +37,6 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) k_tree_attention_tc(const __g
                                                                        const __grid_constant__ SegTable tab,
                                                                        const AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
-  pdl_launch_dependents();
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   AttnCtl* sc = (AttnCtl*)(smem + attn::smem_bytes(DH));
   const int warp = warp_index(), lane = threadIdx.x & 31;
@@ -51,6 +50,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) k_tree_attention_tc(const __g
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_launch_dependents();                 // not before this CTA has its tensor memory
   SPECASR_TRACE_SCOPE(p.tr, SPECASR_KIND_ATTN);
   pdl_wait();
   SPECASR_TRACE_MARK();

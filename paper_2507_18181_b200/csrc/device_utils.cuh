@@ -121,7 +121,10 @@ struct TraceScope {
 #endif
 
 // Programmatic dependent launch (see launch_pdl): wait for the previous kernel of the stream, and let
-// the next one begin its prologue.
+// the next one begin its prologue.  A kernel that runs between two kernels which own tensor memory (norm, rotary, merge)
+// lets the next one begin only after its own wait.  Done at the top, launches ran on ahead without bound: CTA pairs of a
+// projection took SMs and tensor memory while the attention two launches before them was still running, and calls of 65
+// to 128 rows on the 7B shape, whose small grids are resident early, stopped for good now and then.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -220,9 +220,9 @@ __global__ void __launch_bounds__(256) k_rmsnorm_split(const int32_t* __restrict
                                                        bf16* __restrict__ H SPECASR_TRACE_PARAM) {
   namespace cg = cooperative_groups;
   __shared__ float s_ss[kNormCluster];
-  grid_dep_launch();
   SPECASR_TRACE_SCOPE(tr, SPECASR_KIND_NORM);
   cg::cluster_group cluster = cg::this_cluster();
+  cluster.barrier_arrive();                  // waited for below: every CTA of the cluster has started
   const int rank = (int)cluster.block_rank();
   const int row = blockIdx.x / kNormCluster;
   const int tid = threadIdx.x;
@@ -235,6 +235,8 @@ __global__ void __launch_bounds__(256) k_rmsnorm_split(const int32_t* __restrict
     g[it] = kk[it] < k_end ? *reinterpret_cast<const float4*>(gain + kk[it]) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   grid_dep_wait();
+  grid_dep_launch();                         // after the wait: see grid_dep_launch
+  cluster.barrier_wait();
   SPECASR_TRACE_MARK();
   const int status = row < n ? 0 : ctl[CTL_STATUS];   // rows that exist read it behind their data loads (below)
   if (status != 0) return;                   // same for the whole cluster
@@ -333,9 +335,9 @@ __global__ void __launch_bounds__(128) k_rope_append(const __grid_constant__ Seg
                                                      const float2* __restrict__ rope, int layer, bf16* __restrict__ Q,
                                                      size_t q_plane_stride, int page_size, int max_positions
                                                      SPECASR_TRACE_PARAM) {
-  grid_dep_launch();
   SPECASR_TRACE_SCOPE(tr, SPECASR_KIND_ROPE);
   grid_dep_wait();
+  grid_dep_launch();
   SPECASR_TRACE_MARK();
   const int i = blockIdx.x;                    // workspace row
   const SegDev& sg = tab.seg[segment_of_row(tab, i)];
@@ -435,9 +437,9 @@ __global__ void __launch_bounds__(128) k_attn_merge(const __grid_constant__ SegT
                                                     const float2* __restrict__ attML, size_t rows_alloc,
                                                     int Hq, int dh, int n, int rows_total, bf16* __restrict__ AO,
                                                     size_t plane_stride SPECASR_TRACE_PARAM) {
-  grid_dep_launch();
   SPECASR_TRACE_SCOPE(tr, SPECASR_KIND_ATTN_MERGE);
   grid_dep_wait();
+  grid_dep_launch();
   SPECASR_TRACE_MARK();
   if (ctl[CTL_STATUS] != 0) return;
   const int lane = threadIdx.x & 31;

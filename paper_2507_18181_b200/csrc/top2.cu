@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(256) k_top2_probs(const float* __restrict__ lo
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank(), parts = (int)cluster.num_blocks();
   const int row_id = blockIdx.x / parts;
+  cluster.barrier_arrive();                  // waited for before the first write into another CTA: it has started
   grid_dep_launch();
   grid_dep_wait();
   const float* row = logits + (size_t)row_id * vocab;
@@ -90,6 +91,7 @@ __global__ void __launch_bounds__(256) k_top2_probs(const float* __restrict__ lo
   }
   if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = p;
   __syncthreads();
+  cluster.barrier_wait();
   if (threadIdx.x == 0) {
     for (int w = 1; w < 8; ++w) top2_merge(p, s_warp[w]);
     *cluster.map_shared_rank(&s_part[rank], 0) = p;

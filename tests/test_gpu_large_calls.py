@@ -28,3 +28,32 @@ def test_calls_of_more_than_64_rows_match_the_oracle(cfg_name, nodes):
     _check_against_oracle(got, want, tokens, parent)
     again = _verify_gpu(cfg, kv, tokens, parent)
     assert np.array_equal(again["logits"], got["logits"])
+
+
+def test_back_to_back_calls_of_65_to_128_rows_finish_and_repeat():
+    """Calls of this size have small grids between their projections, so launches overlap most.  The 7B geometry cut to two
+    layers, nothing waited for in between: every call must finish with a clean status and repeat its own result."""
+    import torch
+    from paper_2507_18181_b200.runtime import BatchVerifier, DeviceKV, DeviceModel
+    cfg = gen.get_config("7b", n_layers=2, vocab=4096)
+    model = DeviceModel(cfg, gen.WeightStore(cfg, 0))
+    gen_t = torch.Generator("cuda").manual_seed(0)
+    kvs = [DeviceKV(model, max_tokens=1200, max_nodes=256) for _ in range(5)]
+    lens = [611, 697, 728, 876, 1073]
+    for kv, length in zip(kvs, lens):
+        kv.prefill_embeds(torch.randn(length - 87, cfg.d_model, generator=gen_t, device="cuda"))
+        kv.prefill_tokens(torch.randint(0, cfg.vocab, (87,), generator=gen_t, device="cuda", dtype=torch.int32))
+    bv = BatchVerifier(kvs)
+    first = {}
+    for turn in range(60):
+        per = 13 + turn % 13                                   # 65 .. 125 rows
+        torch.manual_seed(per)
+        tokens = torch.randint(0, cfg.vocab, (5 * per,), dtype=torch.int32).cuda()
+        parent = torch.tensor(list(range(-1, per - 1)) * 5, dtype=torch.int32).cuda()
+        bv.verify(tokens, parent, [per * i for i in range(6)])
+        result = torch.cat([bv.out_argmax[:5 * per], bv.out_accept, bv.out_bonus]).clone()
+        if per in first:
+            assert torch.equal(result, first[per])
+        first.setdefault(per, result)
+    torch.cuda.synchronize()
+    assert all(kv.status() == 0 for kv in kvs)
