@@ -42,22 +42,11 @@ namespace {
 constexpr int TILE_M = 128;
 constexpr int SUB_K = 64;               // bf16 elements = 128 bytes = one swizzle row
 constexpr int UMMA_K = 16;
-#ifndef STACK_TM
-#define STACK_TM 1
-#endif
-#ifndef STACK_KSUB
-#define STACK_KSUB 2
-#endif
-// A ring stage holds TM weight tiles (128 rows each) of KSUB 64-wide k sub-blocks and ONE activation block that all
-// of them multiply.  One tile of two sub-blocks (32 KB of weights, contiguous in the tile-packed layout) is what is
-// built.  A tile pair of one sub-block (TM 2, KSUB 1) halves the activation bytes that cross from L2 into shared
-// memory per weight byte, but doubles the k-parts and parked partial sums; it measured 7 % slower at 64 tokens and
-// at 16, and leaving the activation loads out altogether shortens the call by 5 % only: they are not what bounds it.
-constexpr int TM = STACK_TM;
-constexpr int KSUB = STACK_KSUB;
+// A ring stage holds one weight tile (128 rows) of KSUB 64-wide k sub-blocks (16 KB each, contiguous in the tile-packed
+// layout) and the activation block that it multiplies; KSUB is a template parameter of the kernel (see pick_ksub).
+constexpr int TM = 1;                   // weight tiles per stage (pairs measured slower)
 constexpr int W_SUB_BYTES = TILE_M * SUB_K * 2;
-constexpr int W_STAGE_BYTES = TM * KSUB * W_SUB_BYTES;
-constexpr int MAX_STAGES = 6;
+constexpr int MAX_STAGES = 10;
 constexpr int SMEM_LIMIT = 227 * 1024;
 constexpr int WORKERS = 256;            // warps 2..9
 constexpr int NUM_THREADS = 352;        // + TMA weights, MMA, TMA activations
@@ -135,11 +124,12 @@ __device__ __forceinline__ void worker_bar() { asm volatile("bar.sync 1, 256;" :
 // One projection as this CTA sees it.
 struct Gemm {
   const CUtensorMap* tmW;
-  int M, K, KB, Kt, tiles, groups, splits;   // tiles of 128 rows in groups of TM; splits > 0: linear output in `splits` k-parts per group
+  int M, K, KB, Kt, tiles, splits;      // tiles of 128 rows; splits > 0: linear output in `splits` k-parts per tile
   int g_eff;                            // CTAs that take part
-  int U, u0, u1;                        // all (tile group, k-block) units; this CTA's range (whole: no tile is split)
+  int U, u0, u1;                        // all (tile, k-block) units; this CTA's range (whole: no tile is split)
 };
 
+template <int KSUB>
 __device__ __forceinline__ Gemm gemm_of(const StackParams& p, int layer, int which, int cta, int G) {
   Gemm g;
   int whole = 0;
@@ -153,10 +143,9 @@ __device__ __forceinline__ Gemm gemm_of(const StackParams& p, int layer, int whi
   g.KB = (g.K + KSUB * SUB_K - 1) / (KSUB * SUB_K);
   g.Kt = packed_col_tiles(g.K);
   g.tiles = (g.M + TILE_M - 1) / TILE_M;
-  g.groups = (g.tiles + TM - 1) / TM;
-  g.U = g.groups * g.KB;
+  g.U = g.tiles * g.KB;
   if (g.splits > 0) {
-    g.g_eff = g.groups * g.splits;
+    g.g_eff = g.tiles * g.splits;
     if (cta < g.g_eff) {
       const int tile = cta / g.splits, split = cta % g.splits;
       g.u0 = tile * g.KB + split * g.KB / g.splits;
@@ -165,10 +154,10 @@ __device__ __forceinline__ Gemm gemm_of(const StackParams& p, int layer, int whi
       g.u0 = g.u1 = 0;
     }
   } else if (whole) {
-    g.g_eff = g.groups < G ? g.groups : G;
+    g.g_eff = g.tiles < G ? g.tiles : G;
     if (cta < g.g_eff) {
-      g.u0 = cta * g.groups / g.g_eff * g.KB;
-      g.u1 = (cta + 1) * g.groups / g.g_eff * g.KB;
+      g.u0 = cta * g.tiles / g.g_eff * g.KB;
+      g.u1 = (cta + 1) * g.tiles / g.g_eff * g.KB;
     } else {
       g.u0 = g.u1 = 0;
     }
@@ -281,11 +270,12 @@ __device__ __forceinline__ int seg_of_row(const SegTable& tab, int row) {
 #define STACK_TRACE_POINT(point, layer)
 #endif
 
-template <int DH>
+template <int DH, int KSUB>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmAO,
         const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmQ,
         const __grid_constant__ SegTable tab, const StackParams p) {
+  constexpr int W_STAGE_BYTES = KSUB * W_SUB_BYTES;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* ring = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   StackCtl* sc = (StackCtl*)(ring + p.ring_bytes);
@@ -356,8 +346,8 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
           ++c.l;
         }
         Gemm g;
-        if (c.l < p.n_layers) g = gemm_of(p, c.l, phase_of(c.ph), cta, G);
-        else if (p.want_head) g = gemm_of(p, 0, -1, cta, G);
+        if (c.l < p.n_layers) g = gemm_of<KSUB>(p, c.l, phase_of(c.ph), cta, G);
+        else if (p.want_head) g = gemm_of<KSUB>(p, 0, -1, cta, G);
         else {
           c.done = true;
           break;
@@ -450,7 +440,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
       if (gk != -2) {
         // the step before a projection is the one that writes its input
         const CUtensorMap* tmAct = gk == ST_O ? &tmAO : gk == ST_DOWN ? &tmA : &tmH;
-        stream_acts(gemm_of(p, l, gk, cta, G), tmAct, sidx - 1);
+        stream_acts(gemm_of<KSUB>(p, l, gk, cta, G), tmAct, sidx - 1);
       } else if (l < p.n_layers && st == ST_ATTN) {
         if (elect_one()) {
           bool rope_seen = false;
@@ -525,7 +515,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
       const int l = sidx / ST_PER_LAYER, st = sidx - l * ST_PER_LAYER;
       const int gk = gemm_kind_of(l, st, p.n_layers);
       if (gk != -2) {
-        run_gemm(gemm_of(p, l, gk, cta, G));
+        run_gemm(gemm_of<KSUB>(p, l, gk, cta, G));
       } else if (l < p.n_layers && st == ST_ATTN) {
         int L = 0, kc = 0;
 #pragma unroll 1
@@ -1061,13 +1051,13 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
       (void)trace_kind;
       STACK_TRACE_BEGIN();
       if (gk == ST_QKV || gk == ST_O || gk == ST_DOWN) {
-        epi_partial(gemm_of(p, l, gk, cta, G), gk == ST_QKV ? stride_qkv : stride_d);
+        epi_partial(gemm_of<KSUB>(p, l, gk, cta, G), gk == ST_QKV ? stride_qkv : stride_d);
         trace_kind = gk == ST_QKV ? SPECASR_KIND_GEMM_QKV : gk == ST_O ? SPECASR_KIND_GEMM_O : SPECASR_KIND_GEMM_DOWN;
       } else if (gk == ST_GU || gk == -1) {
         wait_step(sidx - 1);                             // the row sums of squares of the norm before it
         STACK_TRACE_MARK();
         load_inv();
-        epi_streamk(gemm_of(p, l, gk, cta, G), gk == ST_GU, p.epoch0 + 1 + l);
+        epi_streamk(gemm_of<KSUB>(p, l, gk, cta, G), gk == ST_GU, p.epoch0 + 1 + l);
         trace_kind = gk == ST_GU ? SPECASR_KIND_GEMM_GU : SPECASR_KIND_GEMM_LM;
       } else if (st == ST_ATTN) {
         attention_step();
@@ -1112,12 +1102,12 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
   }
 }
 
-template <int DH>
+template <int DH, int KSUB>
 cudaError_t launch_dh(const CUtensorMap& tmH, const CUtensorMap& tmAO, const CUtensorMap& tmA, const CUtensorMap& tmQ,
                       const SegTable& tab, const StackParams& p, int grid, size_t smem, cudaStream_t s) {
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_stack<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
+    cudaError_t e = cudaFuncSetAttribute(k_stack<DH, KSUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
     if (e != cudaSuccess) return e;
     configured = true;
   }
@@ -1132,10 +1122,17 @@ cudaError_t launch_dh(const CUtensorMap& tmH, const CUtensorMap& tmAO, const CUt
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_stack<DH>, tmH, tmAO, tmA, tmQ, tab, p);
+  return cudaLaunchKernelEx(&cfg, k_stack<DH, KSUB>, tmH, tmAO, tmA, tmQ, tab, p);
 }
 
 }  // namespace
+
+// 64-wide k sub-blocks per ring stage.  From 48 padded rows on the activations of a stage weigh as much as its weights and
+// the ring holds three stages of two sub-blocks: six or seven finer ones keep more copies in flight (7B shape, 64 rows:
+// 4152 -> 4071 us, 48: 3800 -> 3705; 13B, 64: 7120 -> 6854; 1B, 64: 1005 -> 977).  With fewer rows the ring is four or five
+// stages deep anyway and a stage's hand-offs cost more than they bring (1B, 28 rows: 868 against 880; 0.5B, 8: 966 against
+// 1006), and so they do in a model so narrow that a projection is two stages long (width 256: 91 against 92).
+static int pick_ksub(int n_pad, int d_model) { return n_pad >= 48 && d_model >= 512 ? 1 : 2; }
 
 // Shapes the fused kernel covers: tensor-core attention (head_dim 64 / 128, pages of a multiple of 16 slots),
 // up to 64 token rows (one activation box, both planes in one MMA), key-block count within one counter lane pair.
@@ -1172,7 +1169,8 @@ bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, i
   p.gains = m->gains_dev;
   p.rope = m->rope_table;
   p.n = n_total; p.n_pad = n_pad; p.n_alloc = wk->n_alloc;
-  p.stage_bytes = W_STAGE_BYTES + KSUB * n_pad * 2 * SUB_K * 2;
+  const int ksub = pick_ksub(n_pad, c.d_model), w_stage_bytes = ksub * W_SUB_BYTES;
+  p.stage_bytes = w_stage_bytes + ksub * n_pad * 2 * SUB_K * 2;
   // SiLU * up output tile, or the staged part of a vocabulary tile
   const int epi_bytes = std::max(2 * n_pad * 64 * 2, std::min(n_pad, ARG_TOKENS) * ARG_STRIDE * 4);
   const int attn_bytes = attn::smem_bytes(c.head_dim);
@@ -1184,7 +1182,7 @@ bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, i
   // k parts of the linear projections: tile groups * parts should just fill the SMs
   auto pick_splits = [&](int M, int K) {
     const int groups = (M + TM * TILE_M - 1) / (TM * TILE_M);
-    const int KB = (K + KSUB * SUB_K - 1) / (KSUB * SUB_K);
+    const int KB = (K + ksub * SUB_K - 1) / (ksub * SUB_K);
     int sp = m->n_sm / groups;
     if (sp > kMaxSplitK) sp = kMaxSplitK;
     if (sp > KB) sp = KB;
@@ -1198,8 +1196,8 @@ bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, i
   // SMs idle in the last round, in which the others may still use the whole bandwidth up to what one SM can take in.
   auto whole_tiles = [&](int M, int K) {
     const double kFixupUs = 4.0, kHbm = 7.0e6, kIngest = 15.0e6, kSm = 0.103e6;      // bytes per us
-    const int G = m->n_sm, tiles = (M + TILE_M - 1) / TILE_M, KB = (K + KSUB * SUB_K - 1) / (KSUB * SUB_K);
-    const double all = std::max(W_STAGE_BYTES * G / kHbm, p.stage_bytes * G / kIngest), one = p.stage_bytes / kSm;
+    const int G = m->n_sm, tiles = (M + TILE_M - 1) / TILE_M, KB = (K + ksub * SUB_K - 1) / (ksub * SUB_K);
+    const double all = std::max(w_stage_bytes * G / kHbm, p.stage_bytes * G / kIngest), one = p.stage_bytes / kSm;
     const int rounds = (tiles - 1) / G, rest = tiles - rounds * G;
     const double whole = KB * (rounds * std::max(all, one) + std::max(one, all * rest / G));
     const double ranges = std::max(all * tiles * KB / G, one) + kFixupUs;
@@ -1228,8 +1226,11 @@ bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, i
   const int idx = n_pad / 16 - 1;                         // activation maps are indexed by box rows / 16
   LaunchScope scope(wk, SPECASR_KIND_STACK, s);
   cudaError_t e;                                         // the counters were cleared by the kernel that prepared the rows
-  if (c.head_dim == 64) e = launch_dh<64>(wk->tm_H[idx], wk->tm_AO[idx], wk->tm_A[idx], wk->tm_Q, tab, p, m->n_sm, smem, s);
-  else e = launch_dh<128>(wk->tm_H[idx], wk->tm_AO[idx], wk->tm_A[idx], wk->tm_Q, tab, p, m->n_sm, smem, s);
+  auto launch = [&](auto kernel_launch) {
+    return kernel_launch(wk->tm_H[idx], wk->tm_AO[idx], wk->tm_A[idx], wk->tm_Q, tab, p, m->n_sm, smem, s);
+  };
+  if (c.head_dim == 64) e = ksub == 1 ? launch(launch_dh<64, 1>) : launch(launch_dh<64, 2>);
+  else e = ksub == 1 ? launch(launch_dh<128, 1>) : launch(launch_dh<128, 2>);
   if (e != cudaSuccess) {
     set_error("fused layer stack launch failed: %s", cudaGetErrorString(e));
     return false;
