@@ -538,6 +538,7 @@ static void run_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int
     a.M = m->qkv_dim; a.K = c.d_model; a.epilogue = EPI_PARTIAL;
     run_gemm(wk, a, SPECASR_KIND_GEMM_QKV, s);
     launch_rope_append(wk, tab, n, l, a.splits, s);
+    if (!want_head && l + 1 == c.n_layers) return;   // context fill: K/V of every layer are written, nothing else is read
 #ifdef SPECASR_CROSSCHECK
     if (!att_tc) launch_tree_attention(wk, l, n, tab.splits, s);      // plain kernel, single utterance only
     else
@@ -556,7 +557,6 @@ static void run_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int
     run_gemm(wk, a, SPECASR_KIND_GEMM_DOWN, s);
     pending = a.splits;
   }
-  if (!want_head) return;   // context fill: K/V of every layer are written, the last FFN output is not needed
   launch_rmsnorm_split(wk, ctl_shared, m->g_final, n, n_pad, pending, s);
   a.W = m->lm_head; a.tmW = tc ? &m->tm_lm : nullptr; a.tmAct = wk->tm_H1; a.act = wk->ws.H;
   a.M = c.vocab; a.K = c.d_model; a.epilogue = EPI_ARGMAX; a.amax = wk->ws.amax; a.logits = out_logits;

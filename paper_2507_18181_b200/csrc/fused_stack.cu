@@ -315,7 +315,9 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
   volatile int* abort = &sc->abort;
   int32_t* status = p.ctl + CTL_STATUS;
   const bool live = *(volatile int32_t*)status == 0;
-  const int n_steps = p.n_layers * ST_PER_LAYER + (p.want_head ? 2 : 0);   // final norm and vocabulary projection last
+  // a round ends with the final norm and the vocabulary projection, a context fill with the last layer's K and V: what that
+  // layer would add to the residual stream is not read by anyone
+  const int n_steps = p.want_head ? p.n_layers * ST_PER_LAYER + 2 : (p.n_layers - 1) * ST_PER_LAYER + ST_ROPE + 1;
 
   auto attn_wait = [&](void* bar, uint32_t parity) -> bool { return bar_wait(bar, parity, abort, status); };
 
@@ -346,6 +348,10 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
           ++c.l;
         }
         Gemm g;
+        if (c.l == p.n_layers - 1 && c.ph > 0 && !p.want_head) {
+          c.done = true;
+          break;
+        }
         if (c.l < p.n_layers) g = gemm_of<KSUB>(p, c.l, phase_of(c.ph), cta, G);
         else if (p.want_head) g = gemm_of<KSUB>(p, 0, -1, cta, G);
         else {
