@@ -32,6 +32,7 @@
 // The attention step borrows the ring's shared memory (Q, and a ring of K / V chunks), so the
 // weight producer resumes when the CTA's attention units are done.
 #include <algorithm>
+#include <type_traits>
 
 #include "attention_unit.cuh"
 
@@ -120,6 +121,9 @@ __device__ __forceinline__ void red_relaxed_add(int32_t* p, int v) {
 __device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void worker_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+
+// columns of one of the fixed parts of a residual row
+__host__ __device__ __forceinline__ int norm_part(int d) { return ((d + NORM_PARTS - 1) / NORM_PARTS + 3) & ~3; }
 
 // One projection as this CTA sees it.
 struct Gemm {
@@ -270,7 +274,11 @@ __device__ __forceinline__ int seg_of_row(const SegTable& tab, int row) {
 #define STACK_TRACE_POINT(point, layer)
 #endif
 
-template <int DH, int KSUB>
+// NARROW: half a residual row is at most one group of four columns per worker thread.  Such models have 6 to 12 planes per
+// projection, and their norm and rotary steps are round trips to L2, so they request eight planes at a time instead of four:
+// 0.5B with 8 x 4 rows 978 -> 930 us, 1B chain of 9 839 -> 817.  A template parameter, because the kernel's text is time:
+// with both forms in one kernel the wide models lost 1 to 2 % (7B token 3053 -> 3101; 3065 and 3070 as it stands).
+template <int DH, int KSUB, bool NARROW>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmAO,
         const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmQ,
@@ -594,7 +602,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
     // ---------------- norm step: x += planes, h = x * g as hi / lo planes, sums of squares per half row
     auto norm_step = [&](const float* __restrict__ gain, int n_planes, size_t plane_stride) {
       const int d = p.d;
-      const int d_part = ((d + NORM_PARTS - 1) / NORM_PARTS + 3) & ~3;
+      const int d_part = norm_part(d);
       const int items = p.n * NORM_PARTS;
       const size_t h_plane = (size_t)p.n_alloc * d;
 #pragma unroll 1
@@ -606,25 +614,41 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
 #pragma unroll 1
         for (int k0 = part * d_part + wtid * 4; k0 < k_end; k0 += 2 * WORKERS * 4) {
           const int k1 = k0 + WORKERS * 4;
-          const bool on1 = k1 < k_end;
+          const bool on1 = !NARROW && k1 < k_end;
           float4 v0 = *reinterpret_cast<const float4*>(x + k0);
           float4 v1 = on1 ? *reinterpret_cast<const float4*>(x + k1) : make_float4(0.f, 0.f, 0.f, 0.f);
           const float4 g0 = *reinterpret_cast<const float4*>(gain + k0);
           const float4 g1 = on1 ? *reinterpret_cast<const float4*>(gain + k1) : make_float4(0.f, 0.f, 0.f, 0.f);
+          if constexpr (NARROW) {
 #pragma unroll 1
-          for (int s0 = 0; s0 < n_planes; s0 += 4) {
-            float4 q0[4], q1[4];
+            for (int s0 = 0; s0 < n_planes; s0 += 8) {
+              float4 q[8];
 #pragma unroll
-            for (int s = 0; s < 4; ++s) {
-              const bool on = s0 + s < n_planes;
-              const float* src = p.P + (size_t)(s0 + s) * plane_stride + (size_t)r * d;
-              q0[s] = on ? __ldcg(reinterpret_cast<const float4*>(src + k0)) : make_float4(0.f, 0.f, 0.f, 0.f);
-              q1[s] = (on && on1) ? __ldcg(reinterpret_cast<const float4*>(src + k1)) : make_float4(0.f, 0.f, 0.f, 0.f);
+              for (int s = 0; s < 8; ++s)
+                q[s] = s0 + s < n_planes
+                           ? __ldcg(reinterpret_cast<const float4*>(p.P + (size_t)(s0 + s) * plane_stride + (size_t)r * d + k0))
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+              for (int s = 0; s < 8; ++s) {
+                v0.x += q[s].x; v0.y += q[s].y; v0.z += q[s].z; v0.w += q[s].w;
+              }
             }
+          } else {
+#pragma unroll 1
+            for (int s0 = 0; s0 < n_planes; s0 += 4) {
+              float4 q0[4], q1[4];
 #pragma unroll
-            for (int s = 0; s < 4; ++s) {
-              v0.x += q0[s].x; v0.y += q0[s].y; v0.z += q0[s].z; v0.w += q0[s].w;
-              v1.x += q1[s].x; v1.y += q1[s].y; v1.z += q1[s].z; v1.w += q1[s].w;
+              for (int s = 0; s < 4; ++s) {
+                const bool on = s0 + s < n_planes;
+                const float* src = p.P + (size_t)(s0 + s) * plane_stride + (size_t)r * d;
+                q0[s] = on ? __ldcg(reinterpret_cast<const float4*>(src + k0)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                q1[s] = (on && on1) ? __ldcg(reinterpret_cast<const float4*>(src + k1)) : make_float4(0.f, 0.f, 0.f, 0.f);
+              }
+#pragma unroll
+              for (int s = 0; s < 4; ++s) {
+                v0.x += q0[s].x; v0.y += q0[s].y; v0.z += q0[s].z; v0.w += q0[s].w;
+                v1.x += q1[s].x; v1.y += q1[s].y; v1.z += q1[s].z; v1.w += q1[s].w;
+              }
             }
           }
           if (n_planes > 0) {
@@ -890,9 +914,10 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
         const bool is_v = head >= p.Hq + p.Hkv;
         float4 x1 = make_float4(0.f, 0.f, 0.f, 0.f), x2 = x1;
         float4 cs01 = make_float4(1.f, 0.f, 1.f, 0.f), cs23 = cs01;
-        float4 a1[4], a2[4];
+        constexpr int RB = NARROW ? 8 : 4;               // planes per round trip to L2
+        float4 a1[RB], a2[RB];
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
+        for (int s = 0; s < RB; ++s) {
           const bool on = s < p.splits_qkv;
           a1[s] = on ? __ldcg(reinterpret_cast<const float4*>(p.P + s * pstride + c1)) : make_float4(0.f, 0.f, 0.f, 0.f);
           a2[s] = on ? __ldcg(reinterpret_cast<const float4*>(p.P + s * pstride + c2)) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -907,20 +932,20 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
           cs23 = t[1];
         }
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
+        for (int s = 0; s < RB; ++s) {
           x1.x += a1[s].x; x1.y += a1[s].y; x1.z += a1[s].z; x1.w += a1[s].w;
           x2.x += a2[s].x; x2.y += a2[s].y; x2.z += a2[s].z; x2.w += a2[s].w;
         }
 #pragma unroll 1
-        for (int s0 = 4; s0 < p.splits_qkv; s0 += 4) {
+        for (int s0 = RB; s0 < p.splits_qkv; s0 += RB) {
 #pragma unroll
-          for (int s = 0; s < 4; ++s) {
+          for (int s = 0; s < RB; ++s) {
             const bool on = s0 + s < p.splits_qkv;
             a1[s] = on ? __ldcg(reinterpret_cast<const float4*>(p.P + (s0 + s) * pstride + c1)) : make_float4(0.f, 0.f, 0.f, 0.f);
             a2[s] = on ? __ldcg(reinterpret_cast<const float4*>(p.P + (s0 + s) * pstride + c2)) : make_float4(0.f, 0.f, 0.f, 0.f);
           }
 #pragma unroll
-          for (int s = 0; s < 4; ++s) {
+          for (int s = 0; s < RB; ++s) {
             x1.x += a1[s].x; x1.y += a1[s].y; x1.z += a1[s].z; x1.w += a1[s].w;
             x2.x += a2[s].x; x2.y += a2[s].y; x2.z += a2[s].z; x2.w += a2[s].w;
           }
@@ -1108,12 +1133,12 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
   }
 }
 
-template <int DH, int KSUB>
+template <int DH, int KSUB, bool NARROW>
 cudaError_t launch_dh(const CUtensorMap& tmH, const CUtensorMap& tmAO, const CUtensorMap& tmA, const CUtensorMap& tmQ,
                       const SegTable& tab, const StackParams& p, int grid, size_t smem, cudaStream_t s) {
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_stack<DH, KSUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
+    cudaError_t e = cudaFuncSetAttribute(k_stack<DH, KSUB, NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
     if (e != cudaSuccess) return e;
     configured = true;
   }
@@ -1128,7 +1153,7 @@ cudaError_t launch_dh(const CUtensorMap& tmH, const CUtensorMap& tmAO, const CUt
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_stack<DH, KSUB>, tmH, tmAO, tmA, tmQ, tab, p);
+  return cudaLaunchKernelEx(&cfg, k_stack<DH, KSUB, NARROW>, tmH, tmAO, tmA, tmQ, tab, p);
 }
 
 }  // namespace
@@ -1235,8 +1260,13 @@ bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, i
   auto launch = [&](auto kernel_launch) {
     return kernel_launch(wk->tm_H[idx], wk->tm_AO[idx], wk->tm_A[idx], wk->tm_Q, tab, p, m->n_sm, smem, s);
   };
-  if (c.head_dim == 64) e = ksub == 1 ? launch(launch_dh<64, 1>) : launch(launch_dh<64, 2>);
-  else e = ksub == 1 ? launch(launch_dh<128, 1>) : launch(launch_dh<128, 2>);
+  const bool narrow = norm_part(c.d_model) <= WORKERS * 4;
+  auto pick = [&](auto dh) {
+    constexpr int DH = decltype(dh)::value;
+    if (narrow) return ksub == 1 ? launch(launch_dh<DH, 1, true>) : launch(launch_dh<DH, 2, true>);
+    return ksub == 1 ? launch(launch_dh<DH, 1, false>) : launch(launch_dh<DH, 2, false>);
+  };
+  e = c.head_dim == 64 ? pick(std::integral_constant<int, 64>()) : pick(std::integral_constant<int, 128>());
   if (e != cudaSuccess) {
     set_error("fused layer stack launch failed: %s", cudaGetErrorString(e));
     return false;
