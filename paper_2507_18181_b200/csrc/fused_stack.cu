@@ -22,7 +22,8 @@
 // Work split.  Linear projections (QKV, O, down): weight tiles x k-parts, one CTA each; fp32 partial planes
 // that the consuming step adds in plane order.  Non-linear epilogues (SiLU * up, arg-max): the (tile, k-block)
 // list is cut into equal contiguous ranges, a tile that straddles two ranges is completed through a parked
-// partial and a flag, in CTA order.  All of this is independent of timing, so results are deterministic.
+// partial and a flag, in CTA order; where whole tiles per CTA come out even enough, none is split (launch_fused_stack
+// has the rule).  All of this is independent of timing, so results are deterministic.
 //
 // RMSNorm is split in two: the norm step adds the previous projection's planes to the residual stream,
 // writes x * gain as hi / lo planes and leaves the row's sums of squares (two fixed halves per row); the

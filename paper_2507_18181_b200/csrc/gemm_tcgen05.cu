@@ -14,8 +14,8 @@
 //  - From 129 tokens on ("folded") each CTA holds half of the tokens in both planes; one MMA per plane, N = tokens,
 //    accumulates into the same TMEM columns.  Two accumulator sets fit the 512 columns either way.
 // Measured at 256 rows of the 7B shape (events around each launch): gate/up 139 -> 97 us, down 74 -> 50, QKV 33 -> 29,
-// O 29 -> 25; 256 rows x 4096 x 28672 in two planes is 120 GFLOP, so gate/up now runs at 1.24 PFLOP/s and what bounds
-// it is the tensor pipe (a cuBLAS GEMM on these GPUs does 1.4 to 1.6) plus the tail of the split tiles.
+// O 29 -> 25, and gate/up to 91 since (swiglu_pair); 256 rows x 4096 x 28672 in two planes is 120 GFLOP, so it runs at
+// 1.32 PFLOP/s, what a cuBLAS GEMM sustains on these GPUs under their power limit (1.34; 1.63 in a burst).
 //
 // Scheduling.  The kernel is persistent, one CTA pair per SM pair, over (256-row tile, 64-column k-block) units.
 //  - Linear outputs (QKV, O, down): the k-blocks of every tile are cut into `splits` equal parts, one pair each; it
