@@ -333,8 +333,9 @@ specasr_status specasr_accept_logits_static(const float* logits, int32_t vocab, 
  * Top-2 tokens and their probabilities for every row of a logits matrix (the draft side of the method:
  * Section IV-A truncates a draft where the normalised value of its top-1 token falls below a threshold,
  * Section IV-C branches on the second-ranked token there).
- *   logits    : [device] fp32 [n_rows, vocab], row-major, finite values (e.g. out_logits of
- *               specasr_verify_tree_ex run on the draft model)
+ *   logits    : [device] fp32 [n_rows, vocab], row-major (e.g. out_logits of specasr_verify_tree_ex run on the
+ *               draft model); finite values, or -inf for tokens that the caller has masked (probability 0; a row
+ *               keeps at least one finite value)
  *   out_ids   : [device] int32 [n_rows, 2]  most probable and second most probable token (ties: lower id first;
  *               both entries equal when vocab == 1)
  *   out_probs : [device] fp32 [n_rows, 2]   their probabilities under the softmax over the whole row

@@ -28,11 +28,11 @@ __device__ __forceinline__ float key_value(unsigned long long k) {
   u = (u & 0x80000000u) ? (u & 0x7FFFFFFFu) : ~u;
   return __uint_as_float(u);
 }
-// (m, s) with s = sum of exp(x - m) over the elements seen so far; m = -inf and s = 0 when none
+// (m, s) with s = sum of exp(x - m) over the elements seen so far; m = -inf and s = 0 when none but -inf
 __device__ __forceinline__ void lse_merge(float& m, float& s, float m2, float s2) {
   const float mm = fmaxf(m, m2);
-  if (mm == -INFINITY) return;
-  s = s * expf(m - mm) + s2 * expf(m2 - mm);
+  const float ref = mm > -INFINITY ? mm : 0.f;      // nothing to subtract while both have seen nothing
+  s = s * expf(m - ref) + s2 * expf(m2 - ref);
   m = mm;
 }
 
@@ -71,12 +71,14 @@ __global__ void __launch_bounds__(256) k_top2_probs(const float* __restrict__ lo
     for (int u = 0; u < 8; ++u) x[u] = base + u * 256 < v1 ? row[base + u * 256] : -INFINITY;
 #pragma unroll
     for (int u = 0; u < 8; ++u) top = fmaxf(top, x[u]);
-    p.s *= expf(p.m - top);                 // expf(-inf) = 0 covers the first values
+    // masked values (-inf) count for nothing; while a thread has seen nothing else there is no maximum to subtract
+    const float ref = top > -INFINITY ? top : 0.f;
+    p.s *= expf(p.m - ref);                 // expf(-inf) = 0 covers the first values
     p.m = top;
 #pragma unroll
     for (int u = 0; u < 8; ++u)
       if (base + u * 256 < v1) {
-        p.s += expf(x[u] - top);
+        p.s += expf(x[u] - ref);
         top2_push(p.t, pack_max_key(x[u], (uint32_t)(base + u * 256)));
       }
   }

@@ -44,3 +44,24 @@ def test_top2_and_accept_of_a_logits_matrix(vocab, rows):
     assert np.array_equal(out[0].cpu().numpy(), arg) and a == want["accept_len"] and int(bonus) == want["bonus"]
     path = out[1].cpu().numpy()
     assert list(path[:a + 1]) == list(want["path"]) and np.all(path[a + 1:] == -1)
+
+
+@pytest.mark.parametrize("vocab,cut", [(32000, 28000), (32000, 20000), (32000, 1), (9000, 4000), (4096, 2048), (700, 300)])
+def test_top2_of_rows_with_masked_values(vocab, cut):
+    """-inf as a caller's mask: over the tail, the head (whole slices of a row and whole threads see nothing else), every
+    other value, and all but two.  A masked value has probability 0 and changes nothing else (bound as above)."""
+    rng = np.random.default_rng(cut)
+    logits = (rng.standard_normal((4, vocab)) * 2).astype(np.float32)
+    keep = logits[:, :2].copy()
+    logits[0, max(cut, 2):] = -np.inf
+    logits[1, :vocab - max(cut, 2)] = -np.inf
+    logits[2, ::2] = -np.inf
+    logits[3] = -np.inf
+    logits[3, [cut // 2, vocab - 1]] = keep[3]
+    d = torch.from_numpy(logits).cuda()
+    ids = torch.full((4, 2), -7, dtype=torch.int32, device="cuda")
+    probs = torch.empty(4, 2, device="cuda")
+    B.specasr_top2_probs(d.data_ptr(), 4, vocab, ids.data_ptr(), probs.data_ptr())
+    want_ids, want_probs = O.top2_probs(logits.astype(np.float64))
+    assert np.array_equal(ids.cpu().numpy(), want_ids)
+    assert np.allclose(probs.cpu().numpy(), want_probs, rtol=1e-5, atol=0)
