@@ -38,12 +38,13 @@ __global__ void __launch_bounds__(256) k_logit_keys_static(const float* __restri
   grid_dep_launch();                        // from here on everything before this call in the stream has finished
   const int node = blockIdx.y, chunk = blockIdx.x;
   if (node == 0 && chunk == 0 && threadIdx.x == 0) status[0] = 0;
-  const int v0 = (int)((long long)chunk * vocab / gridDim.x), v1 = (int)((long long)(chunk + 1) * vocab / gridDim.x);
-  const float* row = logits + (size_t)node * vocab;
+  // indices count from the slice's start: a stride past a row's end would pass 2^31 in the widest vocabularies
+  const int v0 = (int)((long long)chunk * vocab / gridDim.x), len = (int)((long long)(chunk + 1) * vocab / gridDim.x) - v0;
+  const float* slice = logits + (size_t)node * vocab + v0;
   unsigned long long best = 0ull;
 #pragma unroll 8
-  for (int v = v0 + threadIdx.x; v < v1; v += 256) {
-    const unsigned long long key = pack_max_key(row[v], (uint32_t)v);
+  for (int k = threadIdx.x; k < len; k += 256) {
+    const unsigned long long key = pack_max_key(slice[k], (uint32_t)(v0 + k));
     best = key > best ? key : best;
   }
 #pragma unroll
@@ -182,7 +183,7 @@ extern "C" specasr_status specasr_accept_logits_static(const float* logits, int3
   // that the second one reads
   int chunks = (4 * 148 + n_nodes - 1) / n_nodes;
   if (chunks > kStaticChunks) chunks = kStaticChunks;
-  if (chunks > (vocab + 1023) / 1024) chunks = (vocab + 1023) / 1024;        // at least four values per thread
+  if (chunks > (vocab - 1) / 1024 + 1) chunks = (vocab - 1) / 1024 + 1;      // at least four values per thread
   launch_pdl(k_logit_keys_static, dim3(chunks, n_nodes), dim3(256), 0, s, logits, vocab, status, keys);
   launch_pdl(k_accept_static, dim3(1), dim3(256), 0, s, status, keys, chunks, tokens, parent_idx, n_nodes, vocab, out_argmax,
              out_accept_len, out_path, out_bonus);

@@ -61,14 +61,15 @@ __global__ void __launch_bounds__(256) k_top2_probs(const float* __restrict__ lo
   cluster.barrier_arrive();                  // waited for before the first write into another CTA: it has started
   grid_dep_launch();
   grid_dep_wait();
-  const float* row = logits + (size_t)row_id * vocab;
-  const int v0 = (int)((long long)rank * vocab / parts), v1 = (int)((long long)(rank + 1) * vocab / parts);
+  // indices count from the slice's start: what a thread reads ahead of a row's end would pass 2^31 in the widest vocabularies
+  const int v0 = (int)((long long)rank * vocab / parts), len = (int)((long long)(rank + 1) * vocab / parts) - v0;
+  const float* slice = logits + (size_t)row_id * vocab + v0;
   Top2Part p{{0ull, 0ull}, -INFINITY, 0.f};
-  for (int base = v0 + threadIdx.x; base < v1; base += 256 * 8) {
+  for (int base = threadIdx.x; base < len; base += 256 * 8) {
     float x[8];
     float top = p.m;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = base + u * 256 < v1 ? row[base + u * 256] : -INFINITY;
+    for (int u = 0; u < 8; ++u) x[u] = base + u * 256 < len ? slice[base + u * 256] : -INFINITY;
 #pragma unroll
     for (int u = 0; u < 8; ++u) top = fmaxf(top, x[u]);
     // masked values (-inf) count for nothing; while a thread has seen nothing else there is no maximum to subtract
@@ -77,9 +78,9 @@ __global__ void __launch_bounds__(256) k_top2_probs(const float* __restrict__ lo
     p.m = top;
 #pragma unroll
     for (int u = 0; u < 8; ++u)
-      if (base + u * 256 < v1) {
+      if (base + u * 256 < len) {
         p.s += expf(x[u] - ref);
-        top2_push(p.t, pack_max_key(x[u], (uint32_t)(base + u * 256)));
+        top2_push(p.t, pack_max_key(x[u], (uint32_t)(v0 + base + u * 256)));
       }
   }
 #pragma unroll

@@ -65,3 +65,23 @@ def test_top2_of_rows_with_masked_values(vocab, cut):
     want_ids, want_probs = O.top2_probs(logits.astype(np.float64))
     assert np.array_equal(ids.cpu().numpy(), want_ids)
     assert np.allclose(probs.cpu().numpy(), want_probs, rtol=1e-5, atol=0)
+
+
+@pytest.mark.parametrize("vocab", [2**31 - 1, 2**31 - 1500])
+def test_widest_vocabularies(vocab):
+    """One row of up to 2^31 - 1 tokens (8.6 GB): a thread's next index passes 2^31 there.  Everything is masked but three
+    values, one in the last place, so that the expected probabilities are those of three numbers."""
+    d = torch.full((vocab,), -float("inf"), device="cuda")
+    at, val = [5, vocab // 2, vocab - 1], [0.25, 1.0, 2.0]
+    for a, v in zip(at, val):
+        d[a] = v
+    ids, probs = torch.empty(1, 2, dtype=torch.int32, device="cuda"), torch.empty(1, 2, device="cuda")
+    B.specasr_top2_probs(d.data_ptr(), 1, vocab, ids.data_ptr(), probs.data_ptr())
+    e = np.exp(np.array(val))
+    assert ids.tolist() == [[at[2], at[1]]]
+    assert np.allclose(probs.cpu().numpy(), [[e[2] / e.sum(), e[1] / e.sum()]], rtol=1e-5, atol=0)
+    t, p = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    out = torch.full((4,), -7, dtype=torch.int32, device="cuda")
+    B.specasr_accept_logits_static(d.data_ptr(), vocab, t.data_ptr(), p.data_ptr(), 1, out.data_ptr(), out[1:].data_ptr(),
+                                   out[2:].data_ptr(), out[3:].data_ptr())
+    assert out.tolist() == [vocab - 1, 0, 0, vocab - 1]
