@@ -134,6 +134,7 @@ static specasr_status model_create_impl(const specasr_model_config* cfg, const s
   m->rope_table = nullptr;
   m->w_maps_dev = nullptr;
   m->gains_dev = nullptr;
+  m->proj_pairs = 0;
   for (int l = 0; l < c.n_layers; ++l) {
     if (!w->wqkv[l] || !w->wo[l] || !w->wgu[l] || !w->wd[l] || !w->g_attn[l] || !w->g_ffn[l]) {
       delete m;
@@ -160,6 +161,20 @@ static specasr_status model_create_impl(const specasr_model_config* cfg, const s
     delete m;
     set_error("the tensor-core path needs an sm_100 device (found sm_%d%d)", prop.major, prop.minor);
     return SPECASR_ERR_UNSUPPORTED;
+  }
+  if (c.gemm_path == 0) {
+    e = gemm_tc_setup(m);
+    if (e == cudaSuccess) e = attention_tc_setup();
+    if (e == cudaSuccess) e = fused_stack_setup();
+  }
+#ifdef SPECASR_CROSSCHECK
+  if (e == cudaSuccess) e = attention_plain_setup();
+#endif
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    delete m;
+    set_error("this device does not grant the kernels their shared memory: %s", cudaGetErrorString(e));
+    return SPECASR_ERR_CUDA;
   }
   // rotary table in fp64 on the host: angle = pos * base^(-2k/dh)
   const int half = c.head_dim / 2;

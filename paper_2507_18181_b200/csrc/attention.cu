@@ -173,25 +173,35 @@ __global__ void __launch_bounds__(256) k_tree_attention(const int32_t* __restric
 }
 
 template <int DH>
+constexpr size_t smem_bytes() {
+  return sizeof(float) * (ROWS * (DH + 1) + KC * (DH + 1) + KC * DH + ROWS * (KC + 1));
+}
+
+template <int DH>
 void launch_dh(specasr_kv* kv, int layer, int n, int n_splits, cudaStream_t s) {
   const specasr_model* m = kv->m;
   const specasr_model_config& c = m->cfg;
   const int group = c.n_heads / c.n_kv_heads;
-  const size_t smem = sizeof(float) * (ROWS * (DH + 1) + KC * (DH + 1) + KC * DH + ROWS * (KC + 1));
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_tree_attention<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = true;
-  }
   dim3 grid(c.n_kv_heads, (n * group + ROWS - 1) / ROWS, n_splits);
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)DH);
   LaunchScope scope(kv, SPECASR_KIND_ATTN, s);
-  launch_pdl(k_tree_attention<DH>, grid, dim3(256), smem, s, kv->ws.ctl, kv->ws.Q, (size_t)kv->n_alloc * m->q_dim, kv->k_pool,
+  launch_pdl(k_tree_attention<DH>, grid, dim3(256), smem_bytes<DH>(), s, kv->ws.ctl, kv->ws.Q, (size_t)kv->n_alloc * m->q_dim, kv->k_pool,
                                                kv->v_pool, kv->page_table, kv->n_pages, c.page_size, layer,
                                                c.n_heads, c.n_kv_heads, n, kv->ws.anc, n_splits, scale_log2,
                                                kv->ws.attO, kv->ws.attML, (size_t)kv->n_alloc * c.n_heads);
 }
 }  // namespace
+
+cudaError_t attention_plain_setup() {
+  cudaError_t e = cudaSuccess;
+  auto raise = [&](auto kernel, size_t smem) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  };
+  raise(k_tree_attention<32>, smem_bytes<32>());
+  raise(k_tree_attention<64>, smem_bytes<64>());
+  raise(k_tree_attention<128>, smem_bytes<128>());
+  return e;
+}
 
 void launch_tree_attention(specasr_kv* kv, int layer, int n, int n_splits, cudaStream_t s) {
   switch (kv->m->cfg.head_dim) {

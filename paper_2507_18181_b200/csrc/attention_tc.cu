@@ -125,16 +125,12 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) k_tree_attention_tc(const __g
   }
 }
 
+constexpr size_t smem_total(int dh) { return attn::smem_bytes(dh) + sizeof(AttnCtl) + 1024; }
+
 template <int DH>
 void launch_dh(specasr_kv* wk, const SegTable& t, int layer, cudaStream_t s) {
   const specasr_model* m = wk->m;
   const specasr_model_config& c = m->cfg;
-  const size_t smem = attn::smem_bytes(DH) + sizeof(AttnCtl) + 1024;
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_tree_attention_tc<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = true;
-  }
   AttnParams p;
   memset(&p, 0, sizeof(p));
   p.anc = wk->ws.anc;
@@ -152,10 +148,18 @@ void launch_dh(specasr_kv* wk, const SegTable& t, int layer, cudaStream_t s) {
   p.tr = wk->trace;
 #endif
   LaunchScope scope(wk, SPECASR_KIND_ATTN, s);
-  launch_pdl(k_tree_attention_tc<DH>, dim3(t.units < m->n_sm ? t.units : m->n_sm), dim3(ATTN_THREADS), smem, s, wk->tm_Q, t, p);
+  launch_pdl(k_tree_attention_tc<DH>, dim3(t.units < m->n_sm ? t.units : m->n_sm), dim3(ATTN_THREADS), smem_total(DH), s, wk->tm_Q,
+             t, p);
 }
 
 }  // namespace
+
+cudaError_t attention_tc_setup() {
+  cudaError_t e = cudaFuncSetAttribute(k_tree_attention_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_total(64));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_tree_attention_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_total(128));
+  return e;
+}
 
 bool attention_tc_supported(const specasr_model* m) {
   const specasr_model_config& c = m->cfg;

@@ -1137,12 +1137,6 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
 template <int DH, int KSUB, bool NARROW>
 cudaError_t launch_dh(const CUtensorMap& tmH, const CUtensorMap& tmAO, const CUtensorMap& tmA, const CUtensorMap& tmQ,
                       const SegTable& tab, const StackParams& p, int grid, size_t smem, cudaStream_t s) {
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_stack<DH, KSUB, NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(grid);
@@ -1158,6 +1152,22 @@ cudaError_t launch_dh(const CUtensorMap& tmH, const CUtensorMap& tmAO, const CUt
 }
 
 }  // namespace
+
+cudaError_t fused_stack_setup() {
+  cudaError_t e = cudaSuccess;
+  auto raise = [&](auto kernel) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
+  };
+  raise(k_stack<64, 1, false>);
+  raise(k_stack<64, 1, true>);
+  raise(k_stack<64, 2, false>);
+  raise(k_stack<64, 2, true>);
+  raise(k_stack<128, 1, false>);
+  raise(k_stack<128, 1, true>);
+  raise(k_stack<128, 2, false>);
+  raise(k_stack<128, 2, true>);
+  return e;
+}
 
 // 64-wide k sub-blocks per ring stage.  From 48 padded rows on the activations of a stage weigh as much as its weights and
 // the ring holds three stages of two sub-blocks: six or seven finer ones keep more copies in flight (7B shape, 64 rows:

@@ -468,11 +468,6 @@ EncodeTiledFn get_encode() {
 template <int EPI, bool FOLD>
 void launch_epi(const CUtensorMap& tmW, const CUtensorMap& tmAct, const TcParams& p, int pairs, size_t smem,
                 cudaStream_t s) {
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_proj<EPI, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
-    configured = true;
-  }
   launch_pdl_cluster(k_proj<EPI, FOLD>, dim3(2 * pairs), dim3(64 + EPI_THREADS), 2, smem, s, tmW, tmAct, p);
 }
 
@@ -568,38 +563,44 @@ static int act_map_index(int n_pad) {
   return 0;
 }
 
-// CTA pairs that can be resident at once: one per SM pair where the driver's partition allows it.
-static int tc_pairs(const specasr_model* m) {
-  static int cached[64];
-  int& c = cached[m->device & 63];
-  if (c == 0) {
-    cudaFuncSetAttribute(k_proj<EPI_SWIGLU, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(m->n_sm & ~1);
-    cfg.blockDim = dim3(64 + EPI_THREADS);
-    cfg.dynamicSmemBytes = SMEM_LIMIT;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_proj<EPI_SWIGLU, true>, &cfg) != cudaSuccess || n < 1) {
-      cudaGetLastError();
-      n = 1;
-    }
-    c = n < m->n_sm / 2 ? n : m->n_sm / 2;
+cudaError_t gemm_tc_setup(specasr_model* m) {
+  cudaError_t e = cudaSuccess;
+  auto raise = [&](auto kernel) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
+  };
+  raise(k_proj<EPI_PARTIAL, false>);
+  raise(k_proj<EPI_PARTIAL, true>);
+  raise(k_proj<EPI_SWIGLU, false>);
+  raise(k_proj<EPI_SWIGLU, true>);
+  raise(k_proj<EPI_ARGMAX, false>);
+  raise(k_proj<EPI_ARGMAX, true>);
+  if (e != cudaSuccess) return e;
+  // CTA pairs that can be resident at once: one per SM pair where the driver's partition allows it
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(m->n_sm & ~1);
+  cfg.blockDim = dim3(64 + EPI_THREADS);
+  cfg.dynamicSmemBytes = SMEM_LIMIT;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, k_proj<EPI_SWIGLU, true>, &cfg) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    n = 1;
   }
-  return c;
+  m->proj_pairs = n < m->n_sm / 2 ? n : m->n_sm / 2;
+  return cudaSuccess;
 }
 
 // Number of k parts of the linear projections: tiles * parts should just fill the SM pairs.
 int gemm_tc_pick_splits(const specasr_model* m, int M, int K) {
   const int ptiles = (gemm_tc_tiles(M) + 1) / 2;
   const int KB = (K + SUB_K - 1) / SUB_K;
-  int s = tc_pairs(m) / ptiles;
+  int s = m->proj_pairs / ptiles;
   if (s > kMaxSplitK) s = kMaxSplitK;
   if (s > KB) s = KB;
   if (s < 1) s = 1;
@@ -637,7 +638,7 @@ void launch_gemm_tc(specasr_kv* kv, const GemmArgs& a, int kind, cudaStream_t s)
   p.tr = kv->trace;
   p.kind = kind;
 #endif
-  const int units = p.ptiles * p.KB, resident = tc_pairs(m);
+  const int units = p.ptiles * p.KB, resident = m->proj_pairs;
   const int pairs = a.epilogue == EPI_PARTIAL ? p.ptiles * p.splits : (units < resident ? units : resident);
   const size_t smem = (size_t)stages * stage_bytes + sizeof(SharedCtl) + epi_bytes + 1024;
   const CUtensorMap& act = a.tmAct[act_map_index(a.n_pad)];

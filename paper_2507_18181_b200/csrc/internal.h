@@ -64,6 +64,7 @@ struct specasr_model {
   CUtensorMap* w_maps_dev;  // device copy for the fused layer-stack kernel: [4 * layers + 1] QKV, O, gate/up, down, ..., vocabulary
   const float** gains_dev;  // device array [2 * layers + 1]: attention / FFN norm gains per layer, then the final norm
   int n_sm;
+  int proj_pairs;           // CTA pairs of a projection that can be resident at once (tensor-core path)
 };
 
 struct Workspace {
@@ -241,13 +242,18 @@ void launch_set_len(specasr_kv* kv, int len, cudaStream_t s);
 void launch_commit(specasr_kv* kv, const int32_t* path, const int32_t* accept_len, cudaStream_t s);
 
 // ---- attention.cu (plain FMA) / attention_tc.cu (tcgen05)
+// The *_setup functions raise the shared-memory limit of every kernel that asks for more than 48 KB.  The limit belongs to
+// a kernel on one device, so it is set when a model is created, on that model's device, and not remembered per process.
+cudaError_t attention_plain_setup();
 void launch_tree_attention(specasr_kv* kv, int layer, int n, int n_splits, cudaStream_t s);
+cudaError_t attention_tc_setup();
 bool attention_tc_supported(const specasr_model* m);
 void attention_tc_plan(const specasr_model* m, SegTable* tab, const int* len_upper);   // fills chunk, splits, unit0, units
 bool attention_tc_make_maps(specasr_kv* kv);
 void launch_tree_attention_tc(specasr_kv* wk, const SegTable& t, int layer, cudaStream_t s);
 
 // ---- fused_stack.cu: the whole layer stack as one persistent kernel
+cudaError_t fused_stack_setup();
 bool fused_stack_supported(const specasr_kv* wk, int n_total, bool att_tc);
 size_t fused_stack_sync_bytes(const specasr_model* m);
 bool launch_fused_stack(specasr_model* m, specasr_kv* wk, const SegTable& tab, int n_total,
@@ -278,6 +284,7 @@ struct GemmArgs {
 };
 int gemm_fma_tiles(int M);
 void launch_gemm_fma(specasr_kv* kv, const GemmArgs& a, int kind, cudaStream_t s);
+cudaError_t gemm_tc_setup(specasr_model* m);                  // also finds proj_pairs
 int gemm_tc_tiles(int M);
 size_t gemm_tc_fixup_bytes(const specasr_model* m, int n_alloc);
 int gemm_tc_pad(int n);                                       // rows a call's projections are padded to
