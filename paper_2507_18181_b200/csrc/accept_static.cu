@@ -26,6 +26,7 @@ static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 constexpr int kMaxDevices = 64;
 std::mutex g_static_mutex;
 void* g_static_ptr[kMaxDevices];     // device address of g_static_scratch, per device, filled on first use
+int g_static_sms[kMaxDevices];       // SMs of that device, filled with it
 
 // Arg-max of one slice of one row's vocabulary.  Bound by the stream of the logits; the host picks the number of slices
 // so that rows x slices fill the GPU about four times (64 rows of 32000: 10 slices, 640 blocks of 13 values per thread;
@@ -162,8 +163,9 @@ extern "C" specasr_status specasr_accept_logits_static(const float* logits, int3
     return SPECASR_ERR_CUDA;
   }
   void* base = nullptr;
+  int sms = 0;
   {
-    // first call on this device: look up where the device keeps the array (no allocation happens here)
+    // first call on this device: look up where the device keeps the array and its size (no allocation happens here)
     std::lock_guard<std::mutex> lock(g_static_mutex);
     if (!g_static_ptr[dev]) {
       void* p = nullptr;
@@ -172,16 +174,22 @@ extern "C" specasr_status specasr_accept_logits_static(const float* logits, int3
         set_error("specasr_accept_logits_static: cudaGetSymbolAddress failed: %s", cudaGetErrorString(e));
         return SPECASR_ERR_CUDA;
       }
+      e = cudaDeviceGetAttribute(&g_static_sms[dev], cudaDevAttrMultiProcessorCount, dev);
+      if (e != cudaSuccess) {
+        set_error("specasr_accept_logits_static: cudaDeviceGetAttribute failed: %s", cudaGetErrorString(e));
+        return SPECASR_ERR_CUDA;
+      }
       g_static_ptr[dev] = p;
     }
     base = g_static_ptr[dev];
+    sms = g_static_sms[dev];
   }
   cudaStream_t s = (cudaStream_t)stream;
   int32_t* status = (int32_t*)base;
   unsigned long long* keys = (unsigned long long*)((unsigned char*)base + kStaticCtlBytes);
   // the array keeps whatever the previous call left: the first kernel clears the status word and rewrites the key slots
   // that the second one reads
-  int chunks = (4 * 148 + n_nodes - 1) / n_nodes;
+  int chunks = (4 * sms + n_nodes - 1) / n_nodes;
   if (chunks > kStaticChunks) chunks = kStaticChunks;
   if (chunks > (vocab - 1) / 1024 + 1) chunks = (vocab - 1) / 1024 + 1;      // at least four values per thread
   launch_pdl(k_logit_keys_static, dim3(chunks, n_nodes), dim3(256), 0, s, logits, vocab, status, keys);

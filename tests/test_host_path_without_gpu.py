@@ -98,3 +98,22 @@ for dev in (0, 1):
 print(json.dumps(out))
 """)
     assert got == [True, 7]          # SPECASR_ERR_CUDA
+
+
+def test_accept_slices_follow_the_device(run):
+    """Slices of the vocabulary per row: about four blocks per SM of the device at hand, at most 64 and at most one per 1024
+    tokens, from the smallest to the widest vocabulary."""
+    cases = [(1, 32000), (64, 32000), (256, 32000), (5, 70000), (3, 1), (1, 2**31 - 1)]
+    got = run(f"""
+out = []
+for dev, sms in ((0, 148), (1, 18)):
+    fake.fake_set_device(dev)
+    fake.fake_set_sm_count(dev, sms)
+    for n, vocab in {cases}:
+        at = fake.fake_launches()
+        B.specasr_accept_logits_static(16, vocab, 16, 16, n, 16, 16, 16, 0)
+        out.append(launches(at)[0][1])
+print(json.dumps(out))
+""")
+    want = [[min(-(-4 * sms // n), 64, (vocab - 1) // 1024 + 1), n, 1] for sms in (148, 18) for n, vocab in cases]
+    assert got == want
