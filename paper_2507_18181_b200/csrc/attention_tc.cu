@@ -84,6 +84,9 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) k_tree_attention_tc(const __g
         auto wait = [&](void* bar, uint32_t parity) -> bool { return mbar_wait(bar, parity, abort, status); };
         if (!attn::multiply<DH>(&sc->a, smem, tmem, kc, pos, g, units, wait)) break;
       }
+      attn::drain(&sc->a, pos, g, units, [&](void* bar, uint32_t parity) -> bool {
+        return mbar_wait(bar, parity, abort, tab.seg[0].ctl + CTL_STATUS);
+      });
     }
   } else {
     const int quad = warp & 3, half = (warp - 2) >> 2, row = quad * 32 + lane;

@@ -229,6 +229,19 @@ __device__ __forceinline__ bool multiply(Ctl* c, uint8_t* smem, uint32_t tmem, i
   return true;
 }
 
+// The issuer's end: everything that it has asked the tensor core to signal has arrived.  The soft-max warps wait for the last
+// pv_done, but the ring slot that those values came from is signalled behind it, and an arrival that lands after the CTA has
+// left hits shared memory that belongs to another kernel.  Each wait is the one that a further use of the barrier would begin
+// with; a barrier that was never used passes at once.  (In the fused stack grid-wide steps follow every attention step.)
+template <typename Wait>
+__device__ __forceinline__ void drain(Ctl* c, int pos, int g, int units, Wait&& wait) {
+  bool ok = wait(&c->q_empty, (uint32_t)(units & 1) ^ 1u);
+#pragma unroll 1
+  for (int i = g; i < g + 2 && ok; ++i) ok = wait(&c->pv_done[i & 1], (uint32_t)((i >> 1) & 1) ^ 1u);
+#pragma unroll 1
+  for (int i = pos; i < pos + SLOTS && ok; ++i) ok = wait(&c->empty[i & (SLOTS - 1)], (uint32_t)((i / SLOTS) & 1) ^ 1u);
+}
+
 // ---- soft-max and output (eight warps; warps w and w + 4 share a TMEM lane quadrant and a row's chunks: `half` 0 / 1).
 // Waits return a warp-uniform verdict.  `pos` and `g` as above, counted by every thread.
 struct RowState {

@@ -57,3 +57,23 @@ def test_back_to_back_calls_of_65_to_128_rows_finish_and_repeat():
         first.setdefault(per, result)
     torch.cuda.synchronize()
     assert all(kv.status() == 0 for kv in kvs)
+
+
+@pytest.mark.parametrize("cfg_name,nodes,context", [("tiny", 65, 1), ("tiny", 256, 200), ("small", 70, 40), ("small", 129, 330)])
+def test_attention_kernel_right_behind_and_before_others(cfg_name, nodes, context):
+    """Short calls, whose attention CTAs run one or two units of one or a few chunks and leave at once: every signal of the
+    tensor core has to have landed by then.  Many calls with nothing waited for in between, all equal to the oracle."""
+    import torch
+    cfg, store, model, kv = _gpu_stack(cfg_name, 0, 0, max_tokens=768, max_nodes=256, shuffle=3)
+    W, cache, prompt = _fill_both(cfg, store, kv, context, 2, 0)
+    parent = gen.sparse_tree(nodes, seed=nodes)
+    tokens = gen.fill_tree_tokens(parent, cfg.vocab, seed=1, root_token=int(prompt[-1]))
+    got = _verify_gpu(cfg, kv, tokens, parent)
+    _check_against_oracle(got, O.verify_tree(cfg, W, cache, tokens, parent), tokens, parent)
+    t, p = torch.from_numpy(tokens).cuda(), torch.from_numpy(parent).cuda()
+    logits = torch.empty(40, nodes, cfg.vocab, device="cuda")
+    for turn in range(40):
+        kv.verify(t, p, logits[turn])
+    torch.cuda.synchronize()
+    assert kv.status() == 0
+    assert bool((logits == logits[0]).all()) and np.array_equal(logits[0].cpu().numpy().astype(np.float64), got["logits"])
