@@ -23,7 +23,8 @@
  *    (malformed parent array, token id out of range, cache capacity exceeded with a length the host
  *    does not know yet, a bounded wait that ran out) set the device status word: the remaining
  *    kernels of that call do nothing, out_accept_len receives -1, and specasr_poll_status reports
- *    the code.  Nothing traps, asserts or spins without a limit.
+ *    the code.  Nothing traps or asserts, and no kernel spins without a limit; what the hardware itself orders (the
+ *    kernel before in the stream, the other CTAs of a cluster, an SM's tensor memory) is waited for as it comes.
  *
  * Tree format: tokens[n] and parent_idx[n] with parent_idx[0] = -1 and 0 <= parent_idx[i] < i.
  * Node 0 is the root: the last committed token, whose K/V is not in the cache yet; it is not
@@ -62,7 +63,7 @@ typedef struct specasr_model_config {
   int32_t head_dim;     /* 64 or 128 (32 in the cross-check build variant only) */
   int32_t ffn;          /* SwiGLU inner width */
   int32_t vocab;
-  int32_t page_size;    /* tokens per KV page; a multiple of 16, at most 208 (16 in the reference workload; any
+  int32_t page_size;    /* tokens per KV page; a multiple of 16, at most 208 (16 in the benchmarked workload; any
                            multiple of 8 in the cross-check build variant) */
   int32_t max_positions;/* length of the rotary table = largest position + 1 */
   float rms_eps;

@@ -106,6 +106,7 @@ static specasr_status model_create_impl(const specasr_model_config* cfg, const s
     return SPECASR_ERR_UNSUPPORTED;
   }
 #ifndef SPECASR_CROSSCHECK
+  // (208 slots per page is the interface's limit, not the kernels': they fetch 16 slots at a time and never look at a whole page)
   if (c.gemm_path != 0 || (c.head_dim != 64 && c.head_dim != 128) || c.page_size % 16 != 0 || c.page_size > 208 ||
       c.n_heads / c.n_kv_heads > 128) {
     set_error("specasr_model_create: this library has the tensor-core path only (gemm_path 0, head_dim 64 or 128, "
@@ -491,7 +492,7 @@ static void run_gemm(specasr_kv* kv, GemmArgs& a, int kind, cudaStream_t s) {
 }
 
 #ifdef SPECASR_CROSSCHECK
-// Key blocks of the plain attention kernel over `n` nodes of one utterance.
+// Key ranges of the plain attention kernel over `n` nodes of one utterance.
 static int plain_attention_splits(const specasr_kv* kv, int n) {
   const specasr_model_config& c = kv->m->cfg;
   const int group = c.n_heads / c.n_kv_heads;

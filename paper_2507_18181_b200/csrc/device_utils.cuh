@@ -13,8 +13,9 @@ __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16& hi, __nv_bflo
 }
 
 // 2^x by the special-function unit alone (relative error about 2^-22, denormal results flushed to zero).  exp2f()
-// wraps the same instruction in range handling that the soft-max does not need (its arguments are <= 0 and a result
-// below 2^-126 is as good as zero) and that made up a tenth of the attention step.
+// wraps the same instruction in range handling that the soft-max does not need and that made up a tenth of the attention
+// step: a score exceeds the reference of its row by at most 2^8 (attn::RESCALE), where the instruction is as exact as
+// below, and a result below 2^-126 is as good as zero.
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -122,9 +123,11 @@ struct TraceScope {
 
 // Programmatic dependent launch (see launch_pdl): wait for the previous kernel of the stream, and let
 // the next one begin its prologue.  A kernel that runs between two kernels which own tensor memory (norm, rotary, merge)
-// lets the next one begin only after its own wait.  Done at the top, launches ran on ahead without bound: CTA pairs of a
-// projection took SMs and tensor memory while the attention two launches before them was still running, and calls of 65
-// to 128 rows on the 7B shape, whose small grids are resident early, stopped for good now and then.
+// lets the next one begin only after its own wait, so that at most one such kernel waits behind a running one.  When all of
+// them did it at the top, calls of 65 to 128 rows on the 7B shape, whose small grids are resident early, stopped for good
+// now and then.  The cause was not found: a projection and the attention do not fit one SM's shared memory together, so that
+// neither can wait for the other's tensor memory, and every CTA of a kernel is resident before the next one begins.  The
+// norm's writes into cluster peers that might not have started yet were mended in the same change.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

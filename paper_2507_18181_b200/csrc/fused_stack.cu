@@ -1,7 +1,7 @@
 // The whole layer stack of one verification round as ONE persistent kernel (sm_100a), one CTA per SM.
 //
 // A round is a chain of dependent steps per layer (RMSNorm -> QKV projection -> rotary + cache append -> tree
-// attention -> merge of the key blocks -> O projection -> RMSNorm -> gate/up projection with SiLU * up -> down
+// attention -> merge of the key ranges -> O projection -> RMSNorm -> gate/up projection with SiLU * up -> down
 // projection) followed by the final norm and the vocabulary projection with arg-max.  Run as separate kernels,
 // every step pays a drain of the GPU, a launch, and a refill of the weight pipeline, and HBM idles meanwhile;
 // at 64 tree tokens that was more than half of the time of a layer.  Here the CTAs stay resident for the whole
@@ -11,7 +11,7 @@
 //   * warp 10 fetches the matching activation blocks (hi / lo bf16 planes) once the step that produces them
 //     has finished on every CTA, and is the TMA producer of the attention step;
 //   * one thread of warp 1 issues every tcgen05.mma (projections: weights as the A operand, tokens as N, both
-//     planes in one MMA of N = 2 x tokens; attention: S = Q K^T and O = P V as three hi/lo terms each);
+//     planes in one MMA of N = 2 x tokens; attention: S = Q K^T with all four hi/lo products, O = P V with three);
 //   * warps 2..9 drain TMEM (projection epilogues, softmax) and run the element-wise steps.
 // Steps are separated by a grid-wide arrival counter in global memory instead of kernel boundaries: a CTA
 // adds one when its part of a step is written, and whoever needs the step's output polls the counter (the
@@ -1010,7 +1010,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
       }
     };
 
-    // ---------------- merge of the key blocks, normalisation, hi / lo split for the O projection
+    // ---------------- merge of the key ranges, normalisation, hi / lo split for the O projection
     auto merge_step = [&]() {
       const size_t rows_alloc = (size_t)p.n_alloc * p.Hq;
       const int rows_total = p.n * p.Hq;
@@ -1023,7 +1023,7 @@ k_stack(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtenso
         const float2 none = make_float2(-INFINITY, 0.f);
         const float2 ml0 = lane < n_splits ? __ldcg(p.attML + (size_t)lane * rows_alloc + r) : none;
         const float2 ml1 = lane + 32 < n_splits ? __ldcg(p.attML + (size_t)(lane + 32) * rows_alloc + r) : none;
-        constexpr int MB = 10;                        // partial outputs in flight per round trip to L2 (config 3 has 9 key blocks)
+        constexpr int MB = 10;                        // partial outputs in flight per round trip to L2 (64 rows on 1700 positions of the 7B shape: 8 ranges)
         float4 o[MB];
 #pragma unroll
         for (int u = 0; u < MB; ++u)
@@ -1173,11 +1173,12 @@ cudaError_t fused_stack_setup() {
 // the ring holds three stages of two sub-blocks: six or seven finer ones keep more copies in flight (7B shape, 64 rows:
 // 4152 -> 4071 us, 48: 3800 -> 3705; 13B, 64: 7120 -> 6854; 1B, 64: 1005 -> 977).  With fewer rows the ring is four or five
 // stages deep anyway and a stage's hand-offs cost more than they bring (1B, 28 rows: 868 against 880; 0.5B, 8: 966 against
-// 1006), and so they do in a model so narrow that a projection is two stages long (width 256: 91 against 92).
+// 1006).  Models narrower than 512, whose projections are one to three stages long, keep the coarse stages: the two measured
+// alike there (width 256: 91 and 92 us, within what two runs differ by).
 static int pick_ksub(int n_pad, int d_model) { return n_pad >= 48 && d_model >= 512 ? 1 : 2; }
 
 // Shapes the fused kernel covers: tensor-core attention (head_dim 64 / 128, pages of a multiple of 16 slots),
-// up to 64 token rows (one activation box, both planes in one MMA), key-block count within one counter lane pair.
+// up to 64 token rows (one activation box, both planes in one MMA).
 bool fused_stack_supported(const specasr_kv* wk, int n_total, bool att_tc) {
   const specasr_model* m = wk->m;
   if (m->cfg.gemm_path != 0 || !att_tc || !wk->attn_tc || m->w_maps_dev == nullptr) return false;

@@ -99,7 +99,7 @@ struct specasr_kv {
   const int32_t* page_table;
   int max_pages;
   int max_nodes;
-  int n_alloc;              // max_nodes rounded up to 16
+  int n_alloc;              // workspace rows: max_nodes rounded up to 16, 32, 64, 128 or 256
   Workspace ws;
   // host-side state
   int pending_n;            // nodes of the verify awaiting a commit, 0 = none

@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(128) k_attn_merge(const __grid_constant__ SegT
   const float2 ml0 = lane < n_splits ? __ldcg(attML + (size_t)lane * rows_alloc + row) : none;
   const float2 ml1 = lane + 32 < n_splits ? __ldcg(attML + (size_t)(lane + 32) * rows_alloc + row) : none;
   // The partial outputs are requested whatever their weights turn out to be, the first six right behind the
-  // (max, sum) pairs, so that no load waits for another; an empty key block's output was never written and is
+  // (max, sum) pairs, so that no load waits for another; an empty key range's output was never written and is
   // dropped below.
   constexpr int B6 = 6;
   float4 o[B6];

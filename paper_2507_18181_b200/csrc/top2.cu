@@ -3,8 +3,8 @@
 // drafting stops where the normalised top-1 value falls below a threshold; Section IV-C: the second-ranked
 // token at such a position seeds a side branch).  See include/specasr.h for the contract.
 //
-// One block per row.  Every thread scans a strided part of the row once, keeping its two largest packed
-// (ordered logit, ~token id) keys and an online (max, sum of exp) pair; warps and then the block merge those.
+// One to eight CTAs (a cluster) per row.  Every thread scans a strided part of its CTA's slice once, keeping its two largest
+// packed (ordered logit, ~token id) keys and an online (max, sum of exp) pair; warps, CTAs and the cluster merge those.
 #include <cooperative_groups.h>
 
 #include "internal.h"

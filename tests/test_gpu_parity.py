@@ -86,7 +86,7 @@ CASES = [
     ("small", 1, 150, 9, "sparse64"),
     ("small", 0, 150, 9, "sparse64"),
     ("small", 0, 37, 3, "chain8"),
-    ("small", 0, 100, 5, "sparse40"),     # n not a power of two: several activation boxes per stage
+    ("small", 0, 100, 5, "sparse40"),     # n not a power of two: rows padded to 48
 ]
 
 
@@ -142,7 +142,7 @@ def test_verify_matches_oracle(cfg_name, gemm_path, n_audio, n_prompt, tree):
 
 @pytest.mark.parametrize("page_size", [8, 24, 32, 64, 208])
 def test_page_sizes_and_an_exactly_full_cache(page_size):
-    """Pages of 32 / 64 / 208 slots run the tensor-core attention (one TMA box per page), 8 and 24 the plain one;
+    """Pages of 32 / 64 / 208 slots run the tensor-core attention (16 slots per TMA box), 8 and 24 the plain one;
     the cache is sized so that the tree's last node lands in its last slot."""
     n_audio, n_prompt, n = 150, 6, 40
     L = n_audio + n_prompt - 1
@@ -481,7 +481,7 @@ def test_7b_full_size_properties():
 def test_random_tree_shapes(cfg_name):
     """Seeded random topologies (any parent[i] < i: bushy, stringy, stars) and sizes from 1 to 70 nodes, several
     rounds on one cache with commits in between, so that ragged tile tails, odd page offsets and every padding
-    width (16 / 32 / 64 / 128) are hit."""
+    width (16 / 32 / 48 / 64 in the fused stack, 96 in the separate projections) are hit."""
     cfg, store, model, kv = _gpu_stack(cfg_name, 8, 0, max_tokens=640, max_nodes=128, shuffle=9)
     W, cache, prompt = _fill_both(cfg, store, kv, 45, 4, 8)
     rng = np.random.default_rng(1234)
@@ -529,7 +529,7 @@ torch.cuda.synchronize()
 plain = kv.out_argmax[:15].clone()
 rec = kv.trace(lambda: kv.verify(d_t, d_p))
 kinds = [B.KIND_NAMES[int(k) & 0xFF] for k in rec[:, 0]]    # bits 8.. carry layer + 1 for the steps of the fused stack
-# one launch each of prep, embedding and accept; per layer 2 norms, 4 projections, rotary, attention, merge, then the LM head
+# one launch each of prep (with the embedding) and accept; per layer 2 norms, 4 projections, rotary, attention, merge, then the LM head
 assert kinds.count("accept") == 1 and "gemm_lm" in kinds
 for name in ("norm", "gemm_qkv", "rope", "attn", "attn_merge", "gemm_o", "gemm_gu", "gemm_down"):
     assert name in kinds, name

@@ -1,4 +1,4 @@
-"""The four forms of the fused stack's kernel on either side of their rules, against the oracle: residual rows that fill
+"""The forms of the fused stack's kernel on either side of their rules, for both head sizes, against the oracle: residual rows that fill
 one group of four columns per worker thread and half (2048), one group of columns more (2056) and a few only (8-wide
 remainders); the smallest width and row count whose ring stages hold one sub-block (512, 33 rows) and their neighbours."""
 import pytest
@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("d_model,head_dim,nodes", [
-    (2048, 64, 9), (2056, 64, 9), (2048, 128, 3), (2056, 128, 3), (2048, 64, 50), (2056, 128, 50),
+    (2048, 64, 9), (2056, 64, 9), (2048, 128, 3), (2056, 128, 3), (2048, 64, 50), (2056, 64, 50), (2056, 128, 50),
     (512, 64, 32), (512, 64, 33), (504, 64, 33), (1032, 128, 64),
 ])
 def test_forms_of_the_stack_match_the_oracle(d_model, head_dim, nodes):

@@ -89,7 +89,7 @@ def test_7b_shape_all_32_layers_against_the_oracle():
 @pytest.mark.parametrize("n_nodes,chain,kv_len", [(256, False, 4096), (256, False, 512), (34, True, 4096)])
 def test_7b_head_geometry_at_the_corners_of_the_sweep(n_nodes, chain, kv_len):
     """256-node trees (the folded projection path, two accumulator sets) on a short and a long cache, and a chain of
-    33 drafts (padded to 64 rows) on 4096 positions, where the key blocks of the attention no longer fit one wave."""
+    33 drafts (34 rows, padded to 48) on 4096 positions: attention ranges of 34, 6 and 8 chunks of 64 keys."""
     cfg = gen.get_config("7b", n_layers=2)
     parent = gen.chain_tree(n_nodes - 1) if chain else gen.sparse_tree(n_nodes, seed=3)
     n_text = 33
