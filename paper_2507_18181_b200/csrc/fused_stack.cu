@@ -1173,8 +1173,8 @@ cudaError_t fused_stack_setup() {
 // the ring holds three stages of two sub-blocks: six or seven finer ones keep more copies in flight (7B shape, 64 rows:
 // 4152 -> 4071 us, 48: 3800 -> 3705; 13B, 64: 7120 -> 6854; 1B, 64: 1005 -> 977).  With fewer rows the ring is four or five
 // stages deep anyway and a stage's hand-offs cost more than they bring (1B, 28 rows: 868 against 880; 0.5B, 8: 966 against
-// 1006).  Models narrower than 512, whose projections are one to three stages long, keep the coarse stages: the two measured
-// alike there (width 256: 91 and 92 us, within what two runs differ by).
+// 1006), and so they do in models narrower than 512, whose projections are a few stages long (two layers, 40 rows, width
+// 256: 87.3 us coarse, 88.0 fine; 384: 90.7, 92.7; 504: 93.6, 94.4; equal code differed by up to 0.4 us between builds).
 static int pick_ksub(int n_pad, int d_model) { return n_pad >= 48 && d_model >= 512 ? 1 : 2; }
 
 // Shapes the fused kernel covers: tensor-core attention (head_dim 64 / 128, pages of a multiple of 16 slots),

@@ -77,3 +77,21 @@ def test_attention_kernel_right_behind_and_before_others(cfg_name, nodes, contex
     torch.cuda.synchronize()
     assert kv.status() == 0
     assert bool((logits == logits[0]).all()) and np.array_equal(logits[0].cpu().numpy().astype(np.float64), got["logits"])
+
+
+@pytest.mark.parametrize("nodes", [1, 17, 40, 64])
+def test_few_rows_of_a_model_too_wide_for_the_fused_stack(nodes):
+    """A QKV projection of more row tiles than SMs (100 heads of 64: 150 tiles) keeps a call out of the fused stack whatever
+    its rows: the separate kernels run it with 16, 32 or 64 padded rows."""
+    from paper_2507_18181_b200.runtime import DeviceKV, DeviceModel
+    cfg = gen.get_config("tiny", n_heads=100, n_kv_heads=100)
+    store = gen.WeightStore(cfg, 0)
+    model = DeviceModel(cfg, store)
+    kv = DeviceKV(model, max_tokens=300, max_nodes=64, shuffle_pages_seed=5, poison=True)
+    W, cache, prompt = _fill_both(cfg, store, kv, 70, 4, 0)
+    parent = gen.sparse_tree(nodes, seed=2) if nodes > 2 else gen.chain_tree(nodes - 1)
+    tokens = gen.fill_tree_tokens(parent, cfg.vocab, seed=3, root_token=int(prompt[-1]))
+    before = kv.launches()
+    got = _verify_gpu(cfg, kv, tokens, parent)
+    assert kv.launches() - before > 9 * cfg.n_layers
+    _check_against_oracle(got, O.verify_tree(cfg, W, cache, tokens, parent), tokens, parent)
