@@ -78,11 +78,12 @@ def algorithmic_flops(cfg, L, n):
 # profiles/k_stack_config3.md: the 2-layer and the 4-layer cut of config 3 (7B shape, 64 tokens, KV 1700).  Traffic
 # grows by a fixed amount per layer, so a full launch is the 2-layer figure plus (layers - 2) times the per-layer
 # difference.  Valid only for the kernel source it was taken on.
-STACK_TRAFFIC_MB = {"cut2": 1252.6, "cut4": 2228.0}
+STACK_TRAFFIC_MB = {"cut2": 1250.5, "cut4": 2221.2}
 STACK_TRAFFIC_SOURCE_SHA256 = {
-    "fused_stack.cu": "077073dfca1a59de599181e079301eaf000d98cb0b6fb51e392c4d8b4cd71ab5",
-    "sm100_ptx.cuh": "f811f56641d5fa39c0c575ce57fecebd5da4265ce577e5678d955814594e3f4d",
-    "device_utils.cuh": "a35abef135a039a872df2c3961d941f9636495b6918adef1293a236f9905c175",
+    "fused_stack.cu": "7ada71e68561deb76bd645efc148932c11b09fa039648c8704d783f40fd99e48",
+    "attention_unit.cuh": "bff900a2e2da8ed166bb62443b3f4e6fa9494523af7d2bdd3326f524ba0b0325",
+    "sm100_ptx.cuh": "394aad337dda854af423297ce187a4cae139b9fed8db1f0ce86dcefd1f6ebe45",
+    "device_utils.cuh": "1fdc2029bc2e37b678daca7f996420513ee0bbb28e41aaae9d591b0b05a5f42f",
 }
 
 
