@@ -152,7 +152,11 @@ specasr_status specasr_kv_truncate(specasr_kv* kv, int32_t len, void* stream);
 
 /* Context fill (the prefill of Section II-A: audio-embedding vectors followed by prompt text), causal
  * attention, no logits.  embeds [device] fp32 [n, d_model] enter layer 0 directly; tokens [device]
- * int32[n] go through the embedding table.  Any n >= 1 (processed in chunks); advances the length. */
+ * int32[n] go through the embedding table.  Any n >= 1 (processed in chunks); advances the length.
+ * A token id outside the vocabulary sets the status word to SPECASR_ERR_INVALID_TREE; of the call's positions whole groups of
+ * max_nodes before the bad one are kept and counted in the length, the rest are not.
+ * The chunks hold max_nodes positions, or up to three times as many (rounded up to 384 or 768) where the handle is for more than
+ * 64 nodes: a long context is filled several times as fast through such a handle. */
 specasr_status specasr_prefill_embeds(specasr_model* m, specasr_kv* kv, const float* embeds, int32_t n, void* stream);
 specasr_status specasr_prefill_tokens(specasr_model* m, specasr_kv* kv, const int32_t* tokens, int32_t n, void* stream);
 

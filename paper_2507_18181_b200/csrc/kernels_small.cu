@@ -100,7 +100,7 @@ __global__ void k_tree_prep(const __grid_constant__ SegTable tab, const int32_t*
 
 // Context fill: a chunk of n consecutive positions is a chain, i.e. plain causal attention.
 // Only the first chunk of a context-fill call starts from a clean status: a chunk that was refused (capacity, a
-// token id outside the vocabulary) keeps every later chunk of the same call from running on top of the gap.
+// token id outside the vocabulary) keeps every later chunk of the same call from running.
 __global__ void k_chain_prep(int32_t* __restrict__ ctl, int n, int capacity, int first, int32_t* __restrict__ depth,
                              int32_t* __restrict__ pos, unsigned long long* __restrict__ anc, int32_t* __restrict__ sync,
                              int sync_words) {
@@ -108,6 +108,7 @@ __global__ void k_chain_prep(int32_t* __restrict__ ctl, int n, int capacity, int
   grid_dep_launch();
   grid_dep_wait();
   clear_counters(sync, sync_words);
+  if (first && i == 0) ctl[CTL_BAD] = INT_MAX;
   if (!first && ctl[CTL_STATUS] != 0) return;
   const int L = ctl[CTL_LEN];
   if (L < 0 || L + n > capacity) {
@@ -161,21 +162,22 @@ __device__ __forceinline__ int segment_of_row(const SegTable& tab, int row) {
   return b;
 }
 
-// A token id outside [0, vocab) is never turned into an address: the row is skipped and the utterance's status
-// word is set, which turns the rest of the call into no-ops (tree verification has checked the ids before; a
-// context fill has not).
-__global__ void k_embed_tokens(const __grid_constant__ SegTable tab, const int32_t* __restrict__ tokens,
+// A token id outside [0, vocab) is never turned into an address (tree verification has checked the ids before; a context
+// fill has not): its row is zeros, which no earlier position sees, and the first such position of the call is noted.  The chunk
+// runs all the same, because what comes before that position counts (k_advance_len).
+__global__ void k_embed_tokens(int32_t* __restrict__ ctl, const int32_t* __restrict__ tokens, int done,
                                const bf16* __restrict__ E, int d, int vocab, float* __restrict__ X SPECASR_TRACE_PARAM) {
   grid_dep_launch();
   SPECASR_TRACE_SCOPE(tr, SPECASR_KIND_PREP);
   grid_dep_wait();
   SPECASR_TRACE_MARK();
   const int i = blockIdx.x;
-  int32_t* ctl = tab.seg[segment_of_row(tab, i)].ctl;
   if (ctl[CTL_STATUS] != 0) return;
   const int tok = tokens[i];
   if (tok < 0 || tok >= vocab) {
-    if (threadIdx.x == 0) ctl[CTL_STATUS] = SPECASR_ERR_INVALID_TREE;
+    if (threadIdx.x == 0) atomicMin(ctl + CTL_BAD, done + i);
+    for (int k = threadIdx.x * 4; k < d; k += blockDim.x * 4)
+      *reinterpret_cast<float4*>(X + (size_t)i * d + k) = make_float4(0.f, 0.f, 0.f, 0.f);
     return;
   }
   embed_row(E + (size_t)tok * d, d, X + (size_t)i * d);
@@ -191,10 +193,10 @@ __global__ void k_copy_embeds(const int32_t* __restrict__ ctl, const float* __re
     *reinterpret_cast<float4*>(X + (size_t)i * d + k) = *reinterpret_cast<const float4*>(src + (size_t)i * d + k);
 }
 
-void launch_embed_tokens(specasr_kv* wk, const SegTable& t, int n_total, const int32_t* tokens, cudaStream_t s) {
-  LaunchScope scope(wk, SPECASR_KIND_PREP, s);
-  launch_pdl(k_embed_tokens, dim3(n_total), dim3(128), 0, s, t, tokens, wk->m->embed, wk->m->cfg.d_model,
-             wk->m->cfg.vocab, wk->ws.X SPECASR_TRACE_ARG(wk));
+void launch_embed_tokens(specasr_kv* kv, const int32_t* tokens, int n, int done, cudaStream_t s) {
+  LaunchScope scope(kv, SPECASR_KIND_PREP, s);
+  launch_pdl(k_embed_tokens, dim3(n), dim3(128), 0, s, kv->ws.ctl, tokens, done, kv->m->embed, kv->m->cfg.d_model,
+             kv->m->cfg.vocab, kv->ws.X SPECASR_TRACE_ARG(kv));
 }
 
 void launch_copy_embeds(specasr_kv* kv, const float* embeds, int n, cudaStream_t s) {
@@ -638,10 +640,16 @@ void launch_accept(specasr_kv* wk, const SegTable& t, const int32_t* ctl_shared,
 // ------------------------------------------------------------------------------------------------
 // Cache length bookkeeping.
 // `host_len` is the pinned host word from which the host learns the length once the event behind the kernel has passed.
-__global__ void k_advance_len(int32_t* ctl, int n, int32_t* host_len) {
+// A context-fill call keeps whole groups of max_nodes positions in front of a bad token id, however many its chunks hold:
+// `done` positions of the call lie before this one.
+__global__ void k_advance_len(int32_t* ctl, int n, int done, int max_nodes, int32_t* host_len) {
   grid_dep_launch();
   grid_dep_wait();
-  if (ctl[CTL_STATUS] == 0) ctl[CTL_LEN] += n;
+  if (ctl[CTL_STATUS] == 0) {
+    const int bad = ctl[CTL_BAD];
+    ctl[CTL_LEN] += bad == INT_MAX ? n : bad / max_nodes * max_nodes - done;
+    if (bad != INT_MAX) ctl[CTL_STATUS] = SPECASR_ERR_INVALID_TREE;
+  }
   *host_len = ctl[CTL_LEN];
 }
 __global__ void k_set_len(int32_t* ctl, int len) {
@@ -651,9 +659,9 @@ __global__ void k_set_len(int32_t* ctl, int len) {
   ctl[CTL_STATUS] = 0;
   ctl[CTL_N] = 0;
 }
-void launch_advance_len(specasr_kv* kv, int n, cudaStream_t s) {
+void launch_advance_len(specasr_kv* kv, int n, int done, cudaStream_t s) {
   LaunchScope scope(kv, SPECASR_KIND_COMMIT, s);
-  launch_pdl(k_advance_len, dim3(1), dim3(1), 0, s, kv->ws.ctl, n, kv->pinned_dev);
+  launch_pdl(k_advance_len, dim3(1), dim3(1), 0, s, kv->ws.ctl, n, done, kv->max_nodes, kv->pinned_dev);
 }
 void launch_set_len(specasr_kv* kv, int len, cudaStream_t s) {
   LaunchScope scope(kv, SPECASR_KIND_COMMIT, s);

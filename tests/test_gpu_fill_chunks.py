@@ -66,6 +66,40 @@ def test_fill_in_large_chunks_is_as_exact_as_in_chunks_of_256_rows(name, rows):
     assert max(whole) < 2e-5 and all(a <= 1.02 * b for a, b in zip(whole, cut)), (whole, cut)
 
 
+@pytest.mark.parametrize("max_nodes,n,bad,kept", [
+    (256, 800, 700, 512), (256, 800, 500, 256), (256, 1000, 255, 0), (200, 768, 767, 600), (100, 300, 250, 200), (32, 70, 40, 32)])
+def test_a_bad_token_id_keeps_whole_groups_of_max_nodes_positions(max_nodes, n, bad, kept):
+    """... in front of it, in chunks of any size: in a chunk, in the second of two (where the first has to give some back), in the
+    last position, in chunks of max_nodes.  What is kept is what the call without the bad id writes, bit for bit."""
+    from paper_2507_18181_b200 import binding as B
+    from paper_2507_18181_b200.runtime import DeviceKV, DeviceModel
+    cfg = gen.get_config("tiny")
+    store = gen.WeightStore(cfg, 0)
+    model = DeviceModel(cfg, store)
+    good = torch.from_numpy(gen.prompt_tokens(n, cfg.vocab, 0).copy()).cuda()
+    lead = torch.from_numpy(gen.audio_prefix(5, cfg.d_model, 0)).cuda()
+    kv = DeviceKV(model, max_tokens=n + 64, max_nodes=max_nodes, shuffle_pages_seed=4, poison=True)
+    kv.prefill_embeds(lead)
+    kv.prefill_tokens(good)
+    assert kv.status() == 0 and kv.length() == 5 + n
+    want = [kv.read_kv(layer, 5 + n) for layer in range(cfg.n_layers)]
+    for value in (cfg.vocab, -1):
+        tokens = good.clone()
+        tokens[bad:bad + 3] = value
+        kv = DeviceKV(model, max_tokens=n + 64, max_nodes=max_nodes, shuffle_pages_seed=4, poison=True)
+        kv.prefill_embeds(lead)
+        kv.prefill_tokens(tokens)
+        assert kv.status() == B.SPECASR_ERR_INVALID_TREE and kv.length() == 5 + kept
+        for layer in range(cfg.n_layers):
+            for got, all_ in zip(kv.read_kv(layer, 5 + kept), want[layer]):
+                assert np.array_equal(got, all_[:5 + kept])
+    kv.prefill_tokens(good[kept:].contiguous())            # the handle goes on where it stands
+    assert kv.status() == 0 and kv.length() == 5 + n
+    for layer in range(cfg.n_layers):
+        for got, all_ in zip(kv.read_kv(layer, 5 + n), want[layer]):
+            assert np.abs(got - all_).max() < 2e-3
+
+
 def test_fill_does_not_depend_on_earlier_contents():
     """The same fill into a used workspace gives the same cache, bit for bit, after trees and other fills."""
     from paper_2507_18181_b200.runtime import DeviceKV, DeviceModel
