@@ -143,9 +143,10 @@ void launch_dh(specasr_kv* wk, const SegTable& t, int layer, cudaStream_t s) {
   AttnParams p;
   memset(&p, 0, sizeof(p));
   p.anc = wk->ws.anc;
-  p.attO = wk->ws.attO;
-  p.attML = wk->ws.attML;
-  p.rows_alloc = (size_t)(CAUSAL ? wk->n_rows : wk->n_alloc) * c.n_heads;
+  const Workspace& ws = CAUSAL ? wk->fill : wk->ws;
+  p.attO = ws.attO;
+  p.attML = ws.attML;
+  p.rows_alloc = (size_t)ws.rows * c.n_heads;
   p.page_size = c.page_size;
   p.layer = layer;
   p.Hq = c.n_heads;
@@ -260,9 +261,9 @@ bool attention_tc_make_maps(specasr_kv* kv) {
     uint64_t strides[3] = {dh * 2, (uint64_t)m->q_dim * 2, (uint64_t)kv->n_alloc * m->q_dim * 2};
     uint32_t box[4] = {64, (uint32_t)group, (uint32_t)(128 / group), 1};
     if (!make_tensor_map_nd(&kv->tm_Q, kv->ws.Q, 4, dims, strides, box)) return false;
-    dims[2] = (uint64_t)kv->n_rows;
-    strides[2] = (uint64_t)kv->n_rows * m->q_dim * 2;
-    if (!make_tensor_map_nd(&kv->fill_Q, kv->ws.Q, 4, dims, strides, box)) return false;
+    dims[2] = (uint64_t)kv->fill.rows;
+    strides[2] = (uint64_t)kv->fill.rows * m->q_dim * 2;
+    if (kv->fill.rows > 0 && !make_tensor_map_nd(&kv->fill_Q, kv->fill.Q, 4, dims, strides, box)) return false;
   }
   const uint64_t ps = c.page_size;
   // pools: [layer and page and kv head][plane][slot][dh]; box = 64 of dh, 16 slots (any page size is a multiple), both planes

@@ -115,11 +115,9 @@ __global__ void k_chain_prep(int32_t* __restrict__ ctl, int n, int capacity, int
     if (i == 0) ctl[CTL_STATUS] = SPECASR_ERR_KV_CAPACITY;
     return;
   }
-  for (int k = i; k < n; k += blockDim.x) {
-    depth[k] = k;
-    pos[k] = L + k;
-  }
+  for (int k = i; k < n; k += blockDim.x) pos[k] = L + k;
   if (i < n && anc) {
+    depth[i] = i;
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
       const int lo = w * 64;
@@ -148,9 +146,8 @@ void launch_chain_prep(specasr_kv* kv, int n, bool first, cudaStream_t s) {
   int cap = kv->max_pages * m->cfg.page_size;
   if (m->cfg.max_positions < cap) cap = m->cfg.max_positions;
   LaunchScope scope(kv, SPECASR_KIND_PREP, s);
-  launch_pdl(k_chain_prep, dim3(1), dim3(256), 0, s, kv->ws.ctl, n, cap, first ? 1 : 0, kv->ws.depth, kv->ws.pos,
-             n <= kv->n_alloc ? kv->ws.anc : nullptr,              // larger chunks are masked by position (SegTable.causal)
-             kv->ws.sync, (int)(fused_stack_sync_bytes(m) / sizeof(int32_t)));
+  const Workspace& ws = space_of(kv, n);       // larger chunks have no ancestor masks: they are masked by position (SegTable.causal)
+  launch_pdl(k_chain_prep, dim3(1), dim3(256), 0, s, ws.ctl, n, cap, first ? 1 : 0, ws.depth, ws.pos, ws.anc, ws.sync, (int)(fused_stack_sync_bytes(m) / sizeof(int32_t)));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -196,12 +193,12 @@ __global__ void k_copy_embeds(const int32_t* __restrict__ ctl, const float* __re
 void launch_embed_tokens(specasr_kv* kv, const int32_t* tokens, int n, int done, cudaStream_t s) {
   LaunchScope scope(kv, SPECASR_KIND_PREP, s);
   launch_pdl(k_embed_tokens, dim3(n), dim3(128), 0, s, kv->ws.ctl, tokens, done, kv->m->embed, kv->m->cfg.d_model,
-             kv->m->cfg.vocab, kv->ws.X SPECASR_TRACE_ARG(kv));
+             kv->m->cfg.vocab, space_of(kv, n).X SPECASR_TRACE_ARG(kv));
 }
 
 void launch_copy_embeds(specasr_kv* kv, const float* embeds, int n, cudaStream_t s) {
   LaunchScope scope(kv, SPECASR_KIND_PREP, s);
-  launch_pdl(k_copy_embeds, dim3(n), dim3(128), 0, s, kv->ws.ctl, embeds, kv->m->cfg.d_model, kv->ws.X);
+  launch_pdl(k_copy_embeds, dim3(n), dim3(128), 0, s, kv->ws.ctl, embeds, kv->m->cfg.d_model, space_of(kv, n).X);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -312,11 +309,12 @@ void launch_rmsnorm_split(specasr_kv* kv, const int32_t* ctl, const float* gain,
   const specasr_model* m = kv->m;
   const int d = m->cfg.d_model;
   const int d_part = (d + 4 * kNormCluster - 1) / (4 * kNormCluster) * 4;      // columns per CTA, a multiple of 4
-  const size_t stride = (size_t)plane_rows(kv, n) * d;
+  const Workspace& ws = space_of(kv, n);
+  const size_t stride = (size_t)ws.rows * d;
   LaunchScope scope(kv, SPECASR_KIND_NORM, s);
 #define NORM_LAUNCH(I)                                                                                           \
   launch_pdl_cluster(k_rmsnorm_split<I>, dim3(kNormCluster * n_pad), dim3(256), kNormCluster, 0, s, ctl,       \
-                     kv->ws.X, kv->ws.P, n_partials, stride, gain, d, d_part, m->cfg.rms_eps, n, stride, kv->ws.H \
+                     ws.X, ws.P, n_partials, stride, gain, d, d_part, m->cfg.rms_eps, n, stride, ws.H \
                      SPECASR_TRACE_ARG(kv))
   if (d_part <= 1024) NORM_LAUNCH(1);
   else if (d_part <= 2048) NORM_LAUNCH(2);
@@ -425,10 +423,10 @@ void launch_rope_append(specasr_kv* wk, const SegTable& t, int n_total, int laye
   const specasr_model_config& c = m->cfg;
   const int heads_per_block = 128 / (c.head_dim / 8);
   dim3 grid(n_total, (c.n_heads + 2 * c.n_kv_heads + heads_per_block - 1) / heads_per_block);
+  const Workspace& ws = space_of(wk, n_total);
   LaunchScope scope(wk, SPECASR_KIND_ROPE, s);
-  launch_pdl(k_rope_append, grid, dim3(128), 0, s, t, wk->ws.P, n_partials, (size_t)plane_rows(wk, n_total) * m->qkv_dim, m->qkv_dim,
-             c.n_heads, c.n_kv_heads, c.head_dim, wk->ws.pos, m->rope_table, layer, wk->ws.Q,
-             (size_t)plane_rows(wk, n_total) * m->q_dim, c.page_size, c.max_positions SPECASR_TRACE_ARG(wk));
+  launch_pdl(k_rope_append, grid, dim3(128), 0, s, t, ws.P, n_partials, (size_t)ws.rows * m->qkv_dim, m->qkv_dim,
+             c.n_heads, c.n_kv_heads, c.head_dim, ws.pos, m->rope_table, layer, ws.Q, (size_t)ws.rows * m->q_dim, c.page_size, c.max_positions SPECASR_TRACE_ARG(wk));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -514,10 +512,10 @@ __global__ void __launch_bounds__(128) k_attn_merge(const __grid_constant__ SegT
 void launch_attn_merge(specasr_kv* kv, const SegTable& t, const int32_t* ctl, int n, int n_pad, cudaStream_t s) {
   const specasr_model_config& c = kv->m->cfg;
   const int rows_total = n_pad * c.n_heads;
+  const Workspace& ws = space_of(kv, n);
   LaunchScope scope(kv, SPECASR_KIND_ATTN_MERGE, s);
-  launch_pdl(k_attn_merge, dim3((rows_total + 3) / 4), dim3(128), 0, s, t, ctl, kv->ws.attO, kv->ws.attML,
-             (size_t)plane_rows(kv, n) * c.n_heads, c.n_heads, c.head_dim, n, rows_total, kv->ws.AO,
-             (size_t)plane_rows(kv, n) * kv->m->q_dim SPECASR_TRACE_ARG(kv));
+  launch_pdl(k_attn_merge, dim3((rows_total + 3) / 4), dim3(128), 0, s, t, ctl, ws.attO, ws.attML, (size_t)ws.rows * c.n_heads,
+             c.n_heads, c.head_dim, n, rows_total, ws.AO, (size_t)ws.rows * kv->m->q_dim SPECASR_TRACE_ARG(kv));
 }
 
 // ------------------------------------------------------------------------------------------------

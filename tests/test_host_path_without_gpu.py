@@ -117,3 +117,14 @@ print(json.dumps(out))
 """)
     want = [[min(-(-4 * sms // n), 64, (vocab - 1) // 1024 + 1), n, 1] for sms in (148, 18) for n, vocab in cases]
     assert got == want
+
+
+@pytest.mark.parametrize("shape", ["", "head_dim=64, heads=14, kv_heads=2, d=896, ffn=4864, vocab=32000, layers=24",
+                                   "heads=32, kv_heads=8, d=4096, ffn=14336, vocab=32000, layers=32"])
+def test_a_workspace_grows_with_the_nodes_of_a_tree(run, shape):
+    """Twice the nodes, twice the bytes at most: large context-fill chunks live in what a tree has."""
+    got = run(f"""
+m = model({shape})
+print(json.dumps([B.specasr_workspace_bytes(m, n) for n in (16, 32, 64, 128, 256)]))
+""")
+    assert all(a < b <= 2 * a for a, b in zip(got, got[1:])), got
