@@ -616,7 +616,8 @@ int gemm_tc_pick_splits(const specasr_model* m, int M, int K) {
   return s;
 }
 
-// Bytes of the parked-partial workspace for trees of up to n_alloc nodes.
+// Bytes of the parked partial sums of a call of up to n_alloc rows, here and in the fused stack: one tile per CTA, and as much
+// again (the size of a workspace is a known quantity to callers, and larger chunks have tiles of up to twice as many rows).
 size_t gemm_tc_fixup_bytes(const specasr_model* m, int n_alloc) {
   return (size_t)m->n_sm * 2 * n_alloc * TILE_M * sizeof(float);
 }
