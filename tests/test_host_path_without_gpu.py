@@ -128,3 +128,19 @@ m = model({shape})
 print(json.dumps([B.specasr_workspace_bytes(m, n) for n in (16, 32, 64, 128, 256)]))
 """)
     assert all(a < b <= 2 * a for a, b in zip(got, got[1:])), got
+
+
+def test_large_fill_chunks_are_planned_on_devices_of_any_size(run):
+    got = run("""
+out = []
+for dev, sms in ((0, 16), (1, 148), (2, 300)):
+    fake.fake_set_device(dev)
+    fake.fake_set_sm_count(dev, sms)
+    m = model(head_dim=64, heads=14, kv_heads=2, d=896, ffn=4864)
+    kv = cache(m)
+    at = fake.fake_launches()
+    B.specasr_prefill_embeds(m, kv, 16, 750, 0)
+    out.append([grid for _, grid, name in launches(at) if "k_tree_attention" in name])
+print(json.dumps(out))
+""")
+    assert all(len(g) == 1 and 0 < g[0][0] <= sms for g, sms in zip(got, (16, 148, 300))), got
