@@ -2,7 +2,8 @@
 smallest such chunk, the edges of two and three token tiles, two chunks dealt out evenly, a second call on top of the first, a
 workspace of 128 rows (chunks of one token tile and of two), and a gate/up projection of more tiles than SM pairs, whose first
 tiles are dealt out whole, and feed-forward widths that leave a large chunk one plane of partial sums or no room at all,
-and one whose tiles are two parts each on every SM pair (a workspace of 128 rows parks tiles of 256).  Caches against the oracle within 2e-3 (the bar of the other fills), then a tree on top."""
+and one whose tiles are two parts each on every SM pair (a workspace of 128 rows parks tiles of 256), and pages that are no
+power of two.  Caches against the oracle within 2e-3 (the bar of the other fills), then a tree on top."""
 import numpy as np
 import pytest
 import torch
@@ -14,16 +15,16 @@ from test_gpu_parity import _check_against_oracle, _verify_gpu
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("name,over,frames,text,max_nodes", [
+@pytest.mark.parametrize("name,over,frames,text,max_nodes,page_size", [case + (16,) for case in [
     ("tiny", {}, 257, 3, 256), ("tiny", {}, 512, 1, 256), ("tiny", {}, 513, 300, 256), ("tiny", {}, 768, 2, 200),
     ("small", {}, 769, 1, 256), ("tiny", {}, 129, 130, 100), ("tiny", {}, 384, 1, 100), ("tiny", {}, 385, 1, 100),
     ("small", {"ffn": 10240}, 520, 1, 256), ("tiny", {"ffn": 6144}, 520, 1, 256), ("tiny", {"ffn": 8192}, 520, 1, 256),
-    ("tiny", {"ffn": 4736}, 250, 1, 100)])
-def test_fill_in_large_chunks_matches_the_oracle(name, over, frames, text, max_nodes):
+    ("tiny", {"ffn": 4736}, 250, 1, 100)]] + [("tiny", {}, 600, 70, 256, 48), ("small", {}, 300, 1, 256, 208)])
+def test_fill_in_large_chunks_matches_the_oracle(name, over, frames, text, max_nodes, page_size):
     from paper_2507_18181_b200.runtime import DeviceKV, DeviceModel
     cfg = gen.get_config(name, **over)
     store = gen.WeightStore(cfg, 0)
-    model = DeviceModel(cfg, store)
+    model = DeviceModel(cfg, store, page_size=page_size)
     kv = DeviceKV(model, max_tokens=frames + text + 80, max_nodes=max_nodes, shuffle_pages_seed=4, poison=True)
     W = O.Weights(store, cache_layers=True)
     audio = gen.audio_prefix(frames, cfg.d_model, 0)
