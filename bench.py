@@ -78,11 +78,11 @@ def algorithmic_flops(cfg, L, n):
 # profiles/k_stack_config3.md: the 2-layer and the 4-layer cut of config 3 (7B shape, 64 tokens, KV 1700).  Traffic
 # grows by a fixed amount per layer, so a full launch is the 2-layer figure plus (layers - 2) times the per-layer
 # difference.  Valid only for the kernel source it was taken on.
-STACK_TRAFFIC_MB = {"cut2": 1178.8, "cut4": 2096.7}
+STACK_TRAFFIC_MB = {"cut2": 1180.0, "cut4": 2096.8}
 STACK_TRAFFIC_SOURCE_SHA256 = {
     "fused_stack.cu": "ba3f224ffb43a1d0aa88bb9244b1a788a7e5a051016876b8ebde3e6e8e155cd1",
     "attention_unit.cuh": "0050bf072365bdb08902251945a2d9b80665e2f6d762dc2948dbe04d045fa8f7",
-    "sm100_ptx.cuh": "b30442a2a1fad7311f1e07204d52c53255a178ed6795658e968f2d8ae9cd5abb",
+    "sm100_ptx.cuh": "52518df5bf750690a599544dd8449df327c028270d33f0268d90c10f162a5ea6",
     "device_utils.cuh": "8eee227ced46aed899861013d90aa0f6cabb4e4800088727a3804bd3b601b040",
 }
 

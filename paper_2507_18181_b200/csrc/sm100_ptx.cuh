@@ -103,12 +103,12 @@ __device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.al
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
-// L2 policies.  Loads of what a call reads once (weights) ask L2 to drop their lines first.  Without that a layer's weights, three times
-// what L2 holds, push out the partial planes, attention partials and activations that the next step reads: they went to
-// HBM (28 MB of writes per 7B layer at 64 rows) and came back late.  7B, 64 rows: 3970 -> 3775 us, one row 3050 -> 2971,
-// 256 rows 8659 -> 8540; 13B, 64 rows: 6635 -> 6442; 1B, 9 rows: 800 -> 760.  In the fused stack keys and values go the
-// same way and activation blocks, which every SM reads, are kept (7B, 64 rows 3940 -> 3902, 33 on 4063 positions 3808 -> 3759);
-// with more rows several row tiles read the same keys, and dropping them early gained nothing (256 rows 8803, 8845).
+// L2 policies.  Loads of what a call reads once (weights) ask L2 to drop their lines first.  Without that a layer's weights, three
+// times what L2 holds, push out the partial planes, attention partials and activations that the next step reads: they went to
+// HBM (28 MB of writes per 7B layer at 64 rows) and came back late.  Time of a call against loads without a policy, in turn on one
+// GPU: 7B, 64 rows -4.9 %, one row -2.6, 256 rows -1.4; 13B, 64 rows -2.9; 1B, 9 rows -5.  In the fused stack keys and values go the
+// same way and activation blocks, which every SM reads, are kept: 7B, 64 rows another -1.0 %, 33 on 4063 positions -1.3.  With
+// more rows several row tiles read the same keys, and dropping them early gained nothing (7B, 256 rows +0.5 %).
 __device__ __forceinline__ uint64_t make_evict_first() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));

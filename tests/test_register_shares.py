@@ -4,15 +4,18 @@ import os
 import re
 import subprocess
 
+import pytest
+
 from paper_2507_18181_b200 import build
 
 
-def test_shares_add_up_to_what_the_block_is_launched_with(tmp_path):
+@pytest.mark.parametrize("variant", [[], ["-DSPECASR_TRACE"]])
+def test_shares_add_up_to_what_the_block_is_launched_with(tmp_path, variant):
     source = os.path.join(build.HERE, "csrc", "gemm_fill.cu")
     text = open(source).read()
     roles, epilogue = map(int, re.search(r"ROLE_REGS = (\d+), EPI_REGS = (\d+);", text).groups())
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    res = subprocess.run([nvcc, "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-Xptxas", "-v",
+    res = subprocess.run([nvcc, "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-Xptxas", "-v", *variant,
                           "-I", os.path.join(build.ROOT, "include"), "-c", source, "-o", str(tmp_path / "fill.o")],
                          capture_output=True, text=True, check=True)
     used = dict(re.findall(r"Compiling entry function '\w*k_proj_fill\w*ILi(\d)E\w*'.*?Used (\d+) registers", res.stderr,
