@@ -18,7 +18,6 @@ def test_shares_add_up_to_what_the_block_is_launched_with(tmp_path, variant):
     res = subprocess.run([nvcc, "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-Xptxas", "-v", *variant,
                           "-I", os.path.join(build.ROOT, "include"), "-c", source, "-o", str(tmp_path / "fill.o")],
                          capture_output=True, text=True, check=True)
-    used = dict(re.findall(r"Compiling entry function '\w*k_proj_fill\w*ILi(\d)E\w*'.*?Used (\d+) registers", res.stderr,
-                           re.S))
-    assert sorted(used) == ["0", "1", "2"], res.stderr
-    assert 4 * roles + 8 * epilogue <= 12 * int(used["2"])       # mode 2: four warps of roles, eight of the epilogue
+    used = re.findall(r"Compiling entry function '\w*k_proj_fill\w*ILi(\d)ELi\d\w*'.*?Used (\d+) registers", res.stderr, re.S)
+    with_shares = [int(n) for mode, n in used if mode == "2"]       # mode 2: four warps of roles, eight of the epilogue
+    assert with_shares and all(4 * roles + 8 * epilogue <= 12 * n for n in with_shares), res.stderr
